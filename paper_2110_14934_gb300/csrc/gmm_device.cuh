@@ -168,59 +168,16 @@ struct Fields {
     float wc, mur, mug, mub, vc, wd, mud, vd;
 };
 
-// Load / store component i of the pixel whose tile starts at element tb
-// (tile index * 8M * kTile) and sits at column t of it; e0 = tb + t.
-template <int PREC, int M>
-__device__ __forceinline__ Fields load_fields(const void *pl, int64_t e0, int64_t tb, uint32_t t,
-                                              int i) {
-    Fields f;
-    if constexpr (PREC == 0) {
-        const float *b = static_cast<const float *>(pl) + e0 + kFields * i * kTile;
-        f.wc = b[F_WC * kTile];
-        f.mur = b[F_MUR * kTile];
-        f.mug = b[F_MUG * kTile];
-        f.mub = b[F_MUB * kTile];
-        f.vc = b[F_VC * kTile];
-        f.wd = b[F_WD * kTile];
-        f.mud = b[F_MUD * kTile];
-        f.vd = b[F_VD * kTile];
-    } else {
-        const uint2 *g = static_cast<const uint2 *>(pl) + (tb >> 2) + t + 2 * i * kTile;
-        const uint2 g0 = g[0], g1 = g[kTile];
-        f.wc = bf16_lo(g0.x);
-        f.wd = bf16_hi(g0.x);
-        const float2 rg = f16x2_unpack(g0.y), bv = f16x2_unpack(g1.x), dv = f16x2_unpack(g1.y);
-        f.mur = rg.x; f.mug = rg.y;
-        f.mub = bv.x; f.vc = bv.y;
-        f.mud = dv.x; f.vd = dv.y;
-    }
-    return f;
-}
-
-// kDepth: also write w_d and v_d (FP32 stores them separately; FP16 always
-// writes them with their group). sr: nonzero = 32 random bits for the
-// stochastic rounding of the two weights (FP16/BF16 state, kSR builds only).
-template <int PREC, int M, bool kDepth = true, bool kSR = false>
-__device__ __forceinline__ void store_fields(void *pl, int64_t e0, int64_t tb, uint32_t t, int i,
-                                             const Fields &f, uint32_t sr = 0u) {
-    if constexpr (PREC == 0) {
-        float *b = static_cast<float *>(pl) + e0 + kFields * i * kTile;
-        b[F_WC * kTile] = f.wc;
-        b[F_MUR * kTile] = f.mur;
-        b[F_MUG * kTile] = f.mug;
-        b[F_MUB * kTile] = f.mub;
-        b[F_VC * kTile] = f.vc;
-        if (kDepth)
-            b[F_WD * kTile] = f.wd;
-        b[F_MUD * kTile] = f.mud;
-        if (kDepth)
-            b[F_VD * kTile] = f.vd;
-    } else {
-        uint2 *g = static_cast<uint2 *>(pl) + (tb >> 2) + t + 2 * i * kTile;
-        const uint32_t w = (kSR && sr) ? bf16x2_pack_sr(f.wc, f.wd, sr) : bf16x2_pack(f.wc, f.wd);
-        g[0] = make_uint2(w, f16x2_pack_sat(f.mur, f.mug));
-        g[kTile] = make_uint2(f16x2_pack_sat(f.mub, f.vc), f16x2_pack_sat(f.mud, f.vd));
-    }
+// Store component i (FP16/BF16 state) of the pixel in column t of the tile
+// that starts at element tb. sr: nonzero = 32 random bits for the stochastic
+// rounding of the two weights (kSR builds only).
+template <bool kSR>
+__device__ __forceinline__ void store_fields_f16(void *pl, int64_t tb, uint32_t t, int i,
+                                                 const Fields &f, uint32_t sr) {
+    uint2 *g = static_cast<uint2 *>(pl) + (tb >> 2) + t + 2 * i * kTile;
+    const uint32_t w = (kSR && sr) ? bf16x2_pack_sr(f.wc, f.wd, sr) : bf16x2_pack(f.wc, f.wd);
+    g[0] = make_uint2(w, f16x2_pack_sat(f.mur, f.mug));
+    g[kTile] = make_uint2(f16x2_pack_sat(f.mub, f.vc), f16x2_pack_sat(f.mud, f.vd));
 }
 
 // ------------------------------------------------------------ mixture step
@@ -278,22 +235,54 @@ template <> __device__ __forceinline__ void rank_sort<5, 3>(Comp<3> (&c)[5]) { n
 template <> __device__ __forceinline__ void rank_sort<5, 1>(Comp<1> (&c)[5]) { net5(c); }
 template <> __device__ __forceinline__ void rank_sort<5, 4>(Comp<4> (&c)[5]) { net5(c); }
 
+// The same networks on keys with the weights beside them.
+template <int M>
+__device__ __forceinline__ void rank_sort(uint32_t (&key)[M], float (&w)[M]) {
+    auto order = [&](int a, int b) { // a sits before b: the larger key goes first
+        const bool sw = key[b] > key[a];
+        const uint32_t k = sw ? key[b] : key[a];
+        const float x = sw ? w[b] : w[a];
+        key[b] = sw ? key[a] : key[b];
+        w[b] = sw ? w[a] : w[b];
+        key[a] = k;
+        w[a] = x;
+    };
+    if constexpr (M == 3) {
+        order(0, 1); order(0, 2); order(1, 2);
+    } else if constexpr (M == 4) {
+        order(0, 1); order(2, 3); order(0, 2); order(1, 3); order(1, 2);
+    } else {
+        static_assert(M == 5, "3 to 5 components");
+        order(0, 1); order(3, 4); order(2, 4); order(2, 3); order(0, 3); order(0, 2);
+        order(1, 4); order(1, 3); order(1, 2);
+    }
+}
+
 // Background test (§III.A) of the changed component at rank `rank` after
 // the update: it is in B (the shortest rank prefix summing past T) unless the
 // prefix before it already sums past T (prefix sums of non-negative weights
 // do not decrease under rounding, so this equals rank >= B). A miss is
 // foreground.
-template <int M, int D>
-__device__ __forceinline__ int background_test(const Comp<D> (&c)[M], int rank, bool matched,
+template <int M>
+__device__ __forceinline__ int background_test(const float (&w)[M], int rank, bool matched,
                                                float T) {
     float acc = 0.f, before = 0.f;
 #pragma unroll
     for (int r = 0; r < M - 1; ++r) {
-        acc += c[r].w;
+        acc += w[r];
         if (r + 1 == rank)
             before = acc;
     }
     return (!matched || before > T) ? 1 : 0;
+}
+template <int M, int D>
+__device__ __forceinline__ int background_test(const Comp<D> (&c)[M], int rank, bool matched,
+                                               float T) {
+    float w[M];
+#pragma unroll
+    for (int r = 0; r < M; ++r)
+        w[r] = c[r].w;
+    return background_test<M>(w, rank, matched, T);
 }
 
 // The update after the match (§III.A): weights, the changed component's mean
@@ -302,7 +291,7 @@ __device__ __forceinline__ int background_test(const Comp<D> (&c)[M], int rank, 
 // match); d2s: the squared distances. kJ >= 0: every lane of this call
 // matched component kJ (the changed component is then known at compile time
 // and needs no selects); kJ < 0: any outcome.
-template <int M, int D, bool kSkipSorted, bool kOptions, int kJ>
+template <int M, int D, bool kOptions, int kJ>
 __device__ __forceinline__ int mixture_update(Comp<D> (&c)[M], const float (&x)[D],
                                               const StreamPrm &p, uint32_t lanes, uint32_t hit,
                                               const float (&d2s)[M]) {
@@ -388,7 +377,7 @@ __device__ __forceinline__ int mixture_update(Comp<D> (&c)[M], const float (&x)[
     for (int i = 1; i < M; ++i)
         sorted = sorted && !(c[i].key > c[i - 1].key);
     int rank = jj; // the changed component's rank after the update
-    if (!kSkipSorted || __any_sync(lanes, !sorted)) {
+    if (__any_sync(lanes, !sorted)) {
         rank_sort<M, D>(c);
 #pragma unroll
         for (int r = 0; r < M; ++r)
@@ -401,15 +390,13 @@ __device__ __forceinline__ int mixture_update(Comp<D> (&c)[M], const float (&x)[
 }
 
 // One tick of one mixture at one pixel (§III.A). The components are in rank
-// order on entry and on exit. Returns the stream's foreground bit.
-// kSkipSorted: let a warp skip the sorting network when it would change
-// nothing (pays where issue slots, not HBM, bound the kernel); `lanes` is
-// then the set of lanes of the warp that make this same call, computed by
-// the caller before the code diverged (unused otherwise). kFastBest (with
-// kSkipSorted): a path specialised to a match of the best-ranked component
-// when every lane of the call has one (the usual case for background
-// pixels); it computes exactly what the general path does.
-template <int M, int D, bool kSkipSorted, bool kOptions, bool kFastBest = kSkipSorted>
+// order on entry and on exit. Returns the stream's foreground bit. A warp
+// skips the sorting network when it would change nothing; `lanes` is the set
+// of lanes of the warp that make this same call, computed by the caller
+// before the code diverged. Where every lane of the call matches its
+// best-ranked component (the usual case for background pixels) a path
+// specialised to that runs; it computes exactly what the general path does.
+template <int M, int D, bool kOptions>
 __device__ __forceinline__ int mixture_step(Comp<D> (&c)[M], const float (&x)[D],
                                             const StreamPrm &p, uint32_t lanes) {
     // Match: first component, in rank order, within k standard deviations
@@ -428,9 +415,161 @@ __device__ __forceinline__ int mixture_step(Comp<D> (&c)[M], const float (&x)[D]
         if (d2 < p.k2 * c[i].v)
             hit |= 1u << i;
     }
-    if (kSkipSorted && kFastBest && __all_sync(lanes, hit & 1u))
-        return mixture_update<M, D, kSkipSorted, kOptions, 0>(c, x, p, lanes, hit, d2s);
-    return mixture_update<M, D, kSkipSorted, kOptions, -1>(c, x, p, lanes, hit, d2s);
+    if (__all_sync(lanes, hit & 1u))
+        return mixture_update<M, D, kOptions, 0>(c, x, p, lanes, hit, d2s);
+    return mixture_update<M, D, kOptions, -1>(c, x, p, lanes, hit, d2s);
+}
+
+// ------------------------------------------------- mixture step, FP32 state
+// The same tick of one mixture straight on the planes in memory. A tick
+// changes every weight, and of the means and variances only those of the
+// component that matched or was replaced, unless components change places.
+// So it needs every weight and variance (the ranking) and the best-ranked
+// component's mean, loaded by the caller; the other means are loaded only in
+// lanes that do not match the best-ranked component or whose components
+// change places, and only what changed is stored: of 16 M values moved per
+// pixel, 6 M + 10 remain for a background pixel. (Per-lane predicates: a warp
+// moves the 32-byte sectors its lanes ask for. A lane that stores a mean or
+// a variance has loaded that element, so a partly stored sector is one the L2
+// already holds.) The means are never all held in registers: where components
+// change places each plane is permuted on its own. Measured against moving
+// the whole state (HBM-bound at 100% of the copy bandwidth): one 1920x1080
+// camera, M = 5, 101.1 -> 70.1 us per tick (DRAM reads 108 instead of 165
+// bytes per pixel); 64 pooled cameras 2299 -> 1393 us.
+//
+// at(i, k): reference to value k of component i, k = 0 the weight, 1..D the
+// mean, D + 1 the variance. w, v: the weights and variances; mu: the
+// best-ranked component's mean. kJ = 0: every lane of the call matched the
+// best-ranked component.
+template <int M, int D, bool kOptions, int kJ, class At>
+__device__ __forceinline__ int plane_update(At at, float (&w)[M], const float (&v)[M],
+                                            float (&mu)[D], const float (&x)[D],
+                                            const StreamPrm &p, uint32_t lanes, bool matched,
+                                            int j, float d2j) {
+    const int jj = kJ == 0 ? 0 : j;
+    float vj = v[0];
+    if (kJ != 0) {
+#pragma unroll
+        for (int i = 1; i < M; ++i)
+            if (i == jj)
+                vj = v[i];
+    }
+    // Weights: as in mixture_update.
+    float sum = 0.f;
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        float wi = __fmul_rn(w[i], p.oma);
+        if (i == jj)
+            wi = matched ? __fadd_rn(wi, p.alpha) : p.init_w;
+        w[i] = wi;
+        sum = __fadd_rn(sum, wi);
+    }
+    const float inv = __fdividef(1.0f, sum); // within 2 ulp; the sum is near 1
+    if (matched) {
+        float orho = p.oma, rho = p.alpha;
+        if (kOptions)
+            rho = match_rate<D>(p, d2j, vj, orho);
+        float d2n = 0.f;
+#pragma unroll
+        for (int ch = 0; ch < D; ++ch) {
+            mu[ch] = fmaf(orho, mu[ch], rho * x[ch]);
+            const float df = x[ch] - mu[ch];
+            d2n = fmaf(df, df, d2n);
+        }
+        vj = fmaxf(p.v_min, fmaf(orho, vj, rho * (kOptions ? var_sample<D>(p, d2n) : d2n)));
+    } else {
+#pragma unroll
+        for (int ch = 0; ch < D; ++ch)
+            mu[ch] = x[ch];
+        vj = p.init_var;
+    }
+    uint32_t key[M];
+    bool sorted = true;
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        w[i] *= inv;
+        key[i] = rank_key(w[i], i == jj ? vj : v[i], i);
+        if (i > 0)
+            sorted = sorted && !(key[i] > key[i - 1]);
+    }
+    int rank = jj;
+    if (__any_sync(lanes, !sorted)) {
+        // Sort (key, weight); the key's low bits say which component a rank
+        // holds (lanes that are in order keep theirs).
+        rank_sort<M>(key, w);
+        int id[M];
+#pragma unroll
+        for (int r = 0; r < M; ++r) {
+            id[r] = 7 - (int)(key[r] & 7u);
+            if (id[r] == jj)
+                rank = r;
+        }
+#pragma unroll
+        for (int k = 1; k <= D + 1; ++k) {
+            float val[M];
+#pragma unroll
+            for (int r = 0; r < M; ++r) {
+                val[r] = k <= D ? mu[k <= D ? k - 1 : 0] : vj;
+                if (id[r] != r && id[r] != jj)
+                    val[r] = at(id[r], k);
+            }
+#pragma unroll
+            for (int r = 0; r < M; ++r)
+                if (id[r] != r || id[r] == jj)
+                    at(r, k) = val[r];
+        }
+    } else {
+#pragma unroll
+        for (int ch = 0; ch < D; ++ch)
+            at(jj, 1 + ch) = mu[ch];
+        at(jj, D + 1) = vj;
+    }
+#pragma unroll
+    for (int r = 0; r < M; ++r)
+        at(r, 0) = w[r];
+    return background_test<M>(w, rank, matched, p.T);
+}
+
+template <int M, int D, bool kOptions, class At>
+__device__ __forceinline__ int plane_step(At at, float (&w)[M], const float (&v)[M],
+                                          float (&mu)[D], const float (&x)[D],
+                                          const StreamPrm &p, uint32_t lanes) {
+    float d2 = 0.f;
+#pragma unroll
+    for (int ch = 0; ch < D; ++ch) {
+        const float df = x[ch] - mu[ch];
+        d2 = fmaf(df, df, d2);
+    }
+    const bool best = d2 < p.k2 * v[0];
+    if (__all_sync(lanes, best))
+        return plane_update<M, D, kOptions, 0>(at, w, v, mu, x, p, lanes, true, 0, d2);
+    bool matched = best;
+    int jj = 0;
+    if (!best) {
+        jj = M - 1; // replaced on a miss
+        float d2s[M];
+#pragma unroll
+        for (int i = 1; i < M; ++i) {
+            d2s[i] = 0.f;
+#pragma unroll
+            for (int ch = 0; ch < D; ++ch) {
+                const float df = x[ch] - at(i, 1 + ch);
+                d2s[i] = fmaf(df, df, d2s[i]);
+            }
+        }
+#pragma unroll
+        for (int i = M - 1; i >= 1; --i) { // the first match wins
+            if (d2s[i] < p.k2 * v[i]) {
+                matched = true;
+                jj = i;
+                d2 = d2s[i];
+            }
+        }
+#pragma unroll
+        for (int ch = 0; ch < D; ++ch)
+            mu[ch] = at(jj, 1 + ch);
+    }
+    return plane_update<M, D, kOptions, -1>(at, w, v, mu, x, p, lanes, matched, jj, d2);
 }
 
 // List 1 (§III.C) on the low four bits of the per-pixel byte.
@@ -464,36 +603,116 @@ __device__ __forceinline__ uint32_t sr_weights(const CamView &cv, uint32_t p, in
 }
 
 // ------------------------------------------------------------ one pixel
-// p: padded linear pixel index (row * w_pad + x). Returns bit 0 fused label,
-// bit 1 colour foreground, bit 2 depth foreground (all 0 for padding).
-// kVariant: 0 the paper's method with the default readings; 1 the same with
-// the learning-rate and variance options of StreamPrm.flags honoured; 2 the
-// augmentation alternative (options honoured too).
-template <int M, int PREC, bool kSkipSorted, int kVariant>
-__device__ __forceinline__ uint32_t process_pixel(const CamView &cv, int64_t p) {
-    const uint32_t p32 = (uint32_t)p;
-    const uint32_t row = div_wpr(p32 >> 5, cv);
-    const uint32_t x = p32 - row * (uint32_t)cv.w_pad;
-    // Every caller enters with whole warps; the lanes on image pixels (not
-    // row padding) are the ones that run the colour (or augmented) mixture.
-    const uint32_t lanes_c = kSkipSorted ? __ballot_sync(0xffffffffu, x < (uint32_t)cv.W) : 0u;
-    if (x >= (uint32_t)cv.W)
-        return 0u;
-    const int64_t q = (int64_t)row * cv.W + x;
-    const float xc[3] = {(float)cv.rgb[3 * q], (float)cv.rgb[3 * q + 1],
-                         (float)cv.rgb[3 * q + 2]};
-    const uint32_t draw = cv.depth[q];
-    const float xd[1] = {(float)draw};
-    // First element of the pixel's tile, and the pixel's column in it.
-    const int64_t tb = (int64_t)(p32 / kTile) * (kFields * M * kTile);
-    const uint32_t t = p32 % kTile;
-    const int64_t e0 = tb + t;
-    const void *pl = cv.planes;
+// The first tick of a pixel in FP32 state: every component on the sample,
+// w = 1/M; the depth model starts with the first reading (until then its
+// planes are zero). The whole state is written; the foregrounds are 0.
+template <int M, int kVariant>
+__device__ __forceinline__ void first_pixel_f32(const CamView &cv, int64_t p, int64_t e0,
+                                                const float (&xc)[3], uint32_t draw) {
+    const float w0 = 1.0f / (float)M;
+    const bool depth = kVariant != 2 && draw != 0u;
+    float f[kFields];
+    f[F_WC] = w0;
+    f[F_MUR] = xc[0];
+    f[F_MUG] = xc[1];
+    f[F_MUB] = xc[2];
+    f[F_VC] = cv.pc.init_var;
+    f[F_WD] = depth ? w0 : 0.f;
+    f[F_MUD] = kVariant == 2 ? (draw ? cv.depth_scale * (float)draw : 0.f) : (float)draw;
+    f[F_VD] = depth ? cv.pd.init_var : 0.f;
+    float *b = static_cast<float *>(cv.planes) + e0;
+#pragma unroll
+    for (int i = 0; i < M; ++i)
+#pragma unroll
+        for (int k = 0; k < kFields; ++k)
+            b[(kFields * i + k) * kTile] = f[k];
+    cv.fusion[p] = kVariant == 2 ? (uint8_t)0u
+                                 : (uint8_t)fuse_list1(0, 0, depth ? kDepthStarted : 0u);
+}
 
-    if (kVariant == 2) {
+// FP32 state after the first tick. The loads that every lane needs come
+// first, for both mixtures together.
+template <int M, int kVariant>
+__device__ __forceinline__ uint32_t tick_pixel_f32(const CamView &cv, int64_t p, int64_t e0,
+                                                   const float (&xc)[3], uint32_t draw,
+                                                   uint32_t lanes_c) {
+    float *const b = static_cast<float *>(cv.planes) + e0;
+    float w[M], v[M];
+    if constexpr (kVariant == 2) {
         // The augmentation alternative (§III.B): one mixture over R, G, B and
         // the scaled depth, stored in the colour planes plus the depth-mean
         // plane. A zero reading takes the best-ranked component's depth mean.
+        auto at = [b](int i, int k) -> float & {
+            const int f = k < 4 ? F_WC + k : k == 4 ? F_MUD : F_VC;
+            return b[(kFields * i + f) * kTile];
+        };
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            w[i] = at(i, 0);
+            v[i] = at(i, 5);
+        }
+        float mu[4] = {at(0, 1), at(0, 2), at(0, 3), at(0, 4)};
+        const float xa[4] = {xc[0], xc[1], xc[2], draw ? cv.depth_scale * (float)draw : mu[3]};
+        const uint32_t f = (uint32_t)plane_step<M, 4, true>(at, w, v, mu, xa, cv.pc, lanes_c);
+        cv.fusion[p] = (uint8_t)f;
+        return f | (f << 1) | (f << 2);
+    } else {
+        auto at_c = [b](int i, int k) -> float & {
+            return b[(kFields * i + F_WC + k) * kTile];
+        };
+        auto at_d = [b](int i, int k) -> float & {
+            return b[(kFields * i + F_WD + k) * kTile];
+        };
+        float wd[M], vd[M];
+        const uint32_t fb0 = cv.fusion[p];
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            w[i] = at_c(i, 0);
+            v[i] = at_c(i, 4);
+            wd[i] = at_d(i, 0);
+            vd[i] = at_d(i, 2);
+        }
+        float mu[3] = {at_c(0, 1), at_c(0, 2), at_c(0, 3)};
+        float mud[1] = {at_d(0, 1)};
+        const int fgc = plane_step<M, 3, (kVariant != 0)>(at_c, w, v, mu, xc, cv.pc, lanes_c);
+        // The lanes that run the depth mixture: a reading, and a started model.
+        uint32_t fb = fb0;
+        const uint32_t lanes_d = __ballot_sync(lanes_c, draw != 0u && (fb & kDepthStarted));
+        int fgd;
+        if (draw == 0u) {
+            fgd = fgc; // no reading: depth model untouched, depth answer = colour
+        } else if (!(fb & kDepthStarted)) {
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                at_d(i, 0) = 1.0f / (float)M;
+                at_d(i, 1) = (float)draw;
+                at_d(i, 2) = cv.pd.init_var;
+            }
+            fb |= kDepthStarted;
+            fgd = 0;
+        } else {
+            const float xd[1] = {(float)draw};
+            fgd = plane_step<M, 1, (kVariant != 0)>(at_d, wd, vd, mud, xd, cv.pd, lanes_d);
+        }
+        fb = fuse_list1(fgc, fgd, fb);
+        if (fb != fb0)
+            cv.fusion[p] = (uint8_t)fb;
+        return (fb & 1u) | ((uint32_t)fgc << 1) | ((uint32_t)fgd << 2);
+    }
+}
+
+// FP16/BF16 state: every group is loaded, and written back.
+template <int M, int kVariant>
+__device__ __forceinline__ uint32_t tick_pixel_f16(const CamView &cv, int64_t p, int64_t tb,
+                                                   uint32_t t, const float (&xc)[3],
+                                                   uint32_t draw, uint32_t lanes_c) {
+    const float xd[1] = {(float)draw};
+    const uint2 *const g = static_cast<const uint2 *>(cv.planes) + (tb >> 2) + t;
+    auto store = [&](int i, const Fields &f) {
+        const uint32_t sr = kVariant != 0 ? sr_weights(cv, (uint32_t)p, i) : 0u;
+        store_fields_f16<kVariant != 0>(cv.planes, tb, t, i, f, sr);
+    };
+    if (kVariant == 2) {
         Comp<4> a[M];
         float xa[4] = {xc[0], xc[1], xc[2], cv.depth_scale * (float)draw};
         int fg;
@@ -510,31 +729,24 @@ __device__ __forceinline__ uint32_t process_pixel(const CamView &cv, int64_t p) 
         } else {
 #pragma unroll
             for (int i = 0; i < M; ++i) {
-                const Fields f = load_fields<PREC, M>(pl, e0, tb, t, i);
-                a[i].w = f.wc;
-                a[i].mu[0] = f.mur; a[i].mu[1] = f.mug; a[i].mu[2] = f.mub; a[i].mu[3] = f.mud;
-                a[i].v = f.vc;
+                const uint2 g0 = g[2 * i * kTile], g1 = g[(2 * i + 1) * kTile];
+                a[i].w = bf16_lo(g0.x);
+                const float2 rg = f16x2_unpack(g0.y), bv = f16x2_unpack(g1.x);
+                a[i].mu[0] = rg.x; a[i].mu[1] = rg.y; a[i].mu[2] = bv.x;
+                a[i].v = bv.y;
+                a[i].mu[3] = f16x2_unpack(g1.y).x;
             }
             if (draw == 0u)
                 xa[3] = a[0].mu[3];
-            fg = mixture_step<M, 4, kSkipSorted, true, (PREC != 0)>(a, xa, cv.pc, lanes_c);
+            fg = mixture_step<M, 4, true>(a, xa, cv.pc, lanes_c);
         }
-        void *plw = cv.planes;
 #pragma unroll
-        for (int i = 0; i < M; ++i) {
-            // w_d and v_d are unused and read as zero
-            const Fields f = {a[i].w, a[i].mu[0], a[i].mu[1], a[i].mu[2], a[i].v,
-                              0.f,    a[i].mu[3], 0.f};
-            if (PREC != 0 || cv.first)
-                store_fields<PREC, M, true, true>(plw, e0, tb, t, i, f, sr_weights(cv, p32, i));
-            else
-                store_fields<PREC, M, false>(plw, e0, tb, t, i, f);
-        }
+        for (int i = 0; i < M; ++i) // w_d and v_d are unused and read as zero
+            store(i, {a[i].w, a[i].mu[0], a[i].mu[1], a[i].mu[2], a[i].v, 0.f, a[i].mu[3], 0.f});
         const uint32_t f = (uint32_t)fg;
         cv.fusion[p] = (uint8_t)f;
         return f | (f << 1) | (f << 2);
     }
-
     Comp<3> c[M];
     Comp<1> d[M];
     uint32_t fb;
@@ -550,48 +762,31 @@ __device__ __forceinline__ uint32_t process_pixel(const CamView &cv, int64_t p) 
         }
         fgc = 0;
     } else {
+        // The depth values stay packed (two registers per component instead
+        // of three) while the colour mixture runs.
         fb = cv.fusion[p];
-        if constexpr (PREC == 0) {
+        uint32_t dw[M], dmv[M];
 #pragma unroll
-            for (int i = 0; i < M; ++i) {
-                const Fields f = load_fields<PREC, M>(pl, e0, tb, t, i);
-                c[i].w = f.wc;
-                c[i].mu[0] = f.mur; c[i].mu[1] = f.mug; c[i].mu[2] = f.mub;
-                c[i].v = f.vc;
-                d[i].w = f.wd;
-                d[i].mu[0] = f.mud;
-                d[i].v = f.vd;
-            }
-            fgc = mixture_step<M, 3, kSkipSorted, (kVariant != 0), (PREC != 0)>(c, xc, cv.pc, lanes_c);
-        } else {
-            // The depth values stay packed (two registers per component
-            // instead of three) while the colour mixture runs.
-            uint32_t dw[M], dmv[M];
-            const uint2 *g = static_cast<const uint2 *>(pl) + (tb >> 2) + t;
+        for (int i = 0; i < M; ++i) {
+            const uint2 g0 = g[2 * i * kTile], g1 = g[(2 * i + 1) * kTile];
+            c[i].w = bf16_lo(g0.x);
+            const float2 rg = f16x2_unpack(g0.y), bv = f16x2_unpack(g1.x);
+            c[i].mu[0] = rg.x; c[i].mu[1] = rg.y; c[i].mu[2] = bv.x;
+            c[i].v = bv.y;
+            dw[i] = g0.x;
+            dmv[i] = g1.y;
+        }
+        fgc = mixture_step<M, 3, (kVariant != 0)>(c, xc, cv.pc, lanes_c);
 #pragma unroll
-            for (int i = 0; i < M; ++i) {
-                const uint2 g0 = g[2 * i * kTile], g1 = g[(2 * i + 1) * kTile];
-                c[i].w = bf16_lo(g0.x);
-                const float2 rg = f16x2_unpack(g0.y), bv = f16x2_unpack(g1.x);
-                c[i].mu[0] = rg.x; c[i].mu[1] = rg.y; c[i].mu[2] = bv.x;
-                c[i].v = bv.y;
-                dw[i] = g0.x;
-                dmv[i] = g1.y;
-            }
-            fgc = mixture_step<M, 3, kSkipSorted, (kVariant != 0), (PREC != 0)>(c, xc, cv.pc, lanes_c);
-#pragma unroll
-            for (int i = 0; i < M; ++i) {
-                d[i].w = bf16_hi(dw[i]);
-                const float2 mv = f16x2_unpack(dmv[i]);
-                d[i].mu[0] = mv.x;
-                d[i].v = mv.y;
-            }
+        for (int i = 0; i < M; ++i) {
+            d[i].w = bf16_hi(dw[i]);
+            const float2 mv = f16x2_unpack(dmv[i]);
+            d[i].mu[0] = mv.x;
+            d[i].v = mv.y;
         }
     }
-
     // The lanes that run the depth mixture: a reading, and a started model.
-    const uint32_t lanes_d =
-        kSkipSorted ? __ballot_sync(lanes_c, draw != 0u && (fb & kDepthStarted)) : 0u;
+    const uint32_t lanes_d = __ballot_sync(lanes_c, draw != 0u && (fb & kDepthStarted));
     if (draw == 0u) {
         fgd = fgc; // no reading: depth model untouched, depth answer = colour
     } else if (!(fb & kDepthStarted)) {
@@ -604,22 +799,47 @@ __device__ __forceinline__ uint32_t process_pixel(const CamView &cv, int64_t p) 
         fb |= kDepthStarted;
         fgd = 0;
     } else {
-        fgd = mixture_step<M, 1, kSkipSorted, (kVariant != 0), (PREC != 0)>(d, xd, cv.pd, lanes_d);
+        fgd = mixture_step<M, 1, (kVariant != 0)>(d, xd, cv.pd, lanes_d);
     }
     fb = fuse_list1(fgc, fgd, fb);
-
-    void *plw = cv.planes;
 #pragma unroll
-    for (int i = 0; i < M; ++i) {
-        const Fields f = {c[i].w, c[i].mu[0], c[i].mu[1], c[i].mu[2], c[i].v,
-                          d[i].w, d[i].mu[0], d[i].v};
-        if (kVariant == 0)
-            store_fields<PREC, M>(plw, e0, tb, t, i, f);
-        else
-            store_fields<PREC, M, true, true>(plw, e0, tb, t, i, f, sr_weights(cv, p32, i));
-    }
+    for (int i = 0; i < M; ++i)
+        store(i, {c[i].w, c[i].mu[0], c[i].mu[1], c[i].mu[2], c[i].v, d[i].w, d[i].mu[0], d[i].v});
     cv.fusion[p] = (uint8_t)fb;
     return (fb & 1u) | ((uint32_t)fgc << 1) | ((uint32_t)fgd << 2);
+}
+
+// p: padded linear pixel index (row * w_pad + x). Returns bit 0 fused label,
+// bit 1 colour foreground, bit 2 depth foreground (all 0 for padding).
+// kVariant: 0 the paper's method with the default readings; 1 the same with
+// the learning-rate and variance options of StreamPrm.flags honoured; 2 the
+// augmentation alternative (options honoured too).
+template <int M, int PREC, int kVariant>
+__device__ __forceinline__ uint32_t process_pixel(const CamView &cv, int64_t p) {
+    const uint32_t p32 = (uint32_t)p;
+    const uint32_t row = div_wpr(p32 >> 5, cv);
+    const uint32_t x = p32 - row * (uint32_t)cv.w_pad;
+    // Every caller enters with whole warps; the lanes on image pixels (not
+    // row padding) are the ones that run the colour (or augmented) mixture.
+    const uint32_t lanes_c = __ballot_sync(0xffffffffu, x < (uint32_t)cv.W);
+    if (x >= (uint32_t)cv.W)
+        return 0u;
+    const int64_t q = (int64_t)row * cv.W + x;
+    const float xc[3] = {(float)cv.rgb[3 * q], (float)cv.rgb[3 * q + 1],
+                         (float)cv.rgb[3 * q + 2]};
+    const uint32_t draw = cv.depth[q];
+    // First element of the pixel's tile, and the pixel's column in it.
+    const int64_t tb = (int64_t)(p32 / kTile) * (kFields * M * kTile);
+    const uint32_t t = p32 % kTile;
+    if constexpr (PREC == 0) {
+        if (cv.first) {
+            first_pixel_f32<M, kVariant>(cv, p, tb + t, xc, draw);
+            return 0u;
+        }
+        return tick_pixel_f32<M, kVariant>(cv, p, tb + t, xc, draw, lanes_c);
+    } else {
+        return tick_pixel_f16<M, kVariant>(cv, p, tb, t, xc, draw, lanes_c);
+    }
 }
 
 // All 32 lanes of the warp call this for 32 consecutive padded pixels

@@ -2,8 +2,9 @@
 // bit-packed mask, mask packing and confusion counts. (The multi-camera tick
 // is in gmm_pool_kernel.cu.)
 //
-// The tick is HBM-bound: per pixel it reads and writes the whole mixture
-// state (64*M bytes in FP32, 32*M in FP16/BF16) plus 5 bytes of frame, the
+// The tick is a stream over the mixture state: per pixel FP32 state needs
+// about 24 M + 40 bytes of it (what a tick reads and changes, see
+// plane_update), FP16/BF16 state moves all 32 M; plus 5 bytes of frame, the
 // List-1 byte and 1/8 byte of mask. There is no dense contraction, so there
 // is no tensor-core work; the design goal is full-line coalesced traffic
 // with enough bytes in flight per SM.
@@ -37,7 +38,7 @@ __device__ __forceinline__ void tick_body(const CamView &cv) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= cv.n_pad)
         return;
-    const uint32_t bits = process_pixel<M, PREC, PREC != 0, V>(cv, p);
+    const uint32_t bits = process_pixel<M, PREC, V>(cv, p);
     write_mask_words(cv, p >> 5, bits);
 }
 
@@ -56,7 +57,7 @@ __device__ __forceinline__ void tick_body2(const CamView &cv) {
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
         const int64_t p = base + 32 * u + lane;
-        bits[u] = p < cv.n_pad ? process_pixel<M, PREC, PREC != 0, V>(cv, p) : 0u;
+        bits[u] = p < cv.n_pad ? process_pixel<M, PREC, V>(cv, p) : 0u;
     }
 #pragma unroll
     for (int u = 0; u < 2; ++u)
@@ -64,9 +65,9 @@ __device__ __forceinline__ void tick_body2(const CamView &cv) {
             write_mask_words(cv, (base >> 5) + u, bits[u]);
 }
 
-// FP32 state: HBM-bound; the register allocation without a residency hint
-// (64 registers) measured fastest. FP16/BF16 state: issue bound; at least
-// 1024 threads per SM. V: process_pixel's variant (the options are separate
+// FP32 state: latency-bound (64 registers and 32 warps per SM at M = 5; bounds
+// of 48 and 40 registers measured 66 and 70 us against 70 at 1920x1080, but
+// slower for M = 3). FP16/BF16 state: issue bound; at least 1024 threads per SM. V: process_pixel's variant (the options are separate
 // instantiations, so the default kernels carry none of them). Small CTAs
 // measured faster than 256 threads: a CTA's slot frees as soon as its own
 // warps finish. A persistent grid-stride form measured slower (its loop

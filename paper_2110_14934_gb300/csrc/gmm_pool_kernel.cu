@@ -26,7 +26,7 @@ template <int M, int PREC, int V>
 __device__ __forceinline__ void pool_tile(const CamView &cv, int64_t p0, int64_t p1) {
     for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
         // p1 - p0 is a multiple of 32 and blockDim too: warps stay whole.
-        const uint32_t bits = process_pixel<M, PREC, true, V>(cv, p);
+        const uint32_t bits = process_pixel<M, PREC, V>(cv, p);
         write_mask_words(cv, p >> 5, bits);
     }
 }
@@ -190,13 +190,13 @@ __device__ __forceinline__ void flat_chunk(const CamView &cv, int64_t base) {
     const int lane = threadIdx.x & 31;
     if constexpr (PREC == 0) { // n_pad is a multiple of 32: the chunk is whole
         const int64_t p = base + lane;
-        write_mask_words(cv, p >> 5, process_pixel<M, PREC, true, V>(cv, p));
+        write_mask_words(cv, p >> 5, process_pixel<M, PREC, V>(cv, p));
     } else {
         uint32_t bits[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int64_t p = base + 32 * u + lane;
-            bits[u] = p < cv.n_pad ? process_pixel<M, PREC, true, V>(cv, p) : 0u;
+            bits[u] = p < cv.n_pad ? process_pixel<M, PREC, V>(cv, p) : 0u;
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u)
