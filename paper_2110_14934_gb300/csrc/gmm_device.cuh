@@ -235,29 +235,6 @@ template <> __device__ __forceinline__ void rank_sort<5, 3>(Comp<3> (&c)[5]) { n
 template <> __device__ __forceinline__ void rank_sort<5, 1>(Comp<1> (&c)[5]) { net5(c); }
 template <> __device__ __forceinline__ void rank_sort<5, 4>(Comp<4> (&c)[5]) { net5(c); }
 
-// The same networks on keys with the weights beside them.
-template <int M>
-__device__ __forceinline__ void rank_sort(uint32_t (&key)[M], float (&w)[M]) {
-    auto order = [&](int a, int b) { // a sits before b: the larger key goes first
-        const bool sw = key[b] > key[a];
-        const uint32_t k = sw ? key[b] : key[a];
-        const float x = sw ? w[b] : w[a];
-        key[b] = sw ? key[a] : key[b];
-        w[b] = sw ? w[a] : w[b];
-        key[a] = k;
-        w[a] = x;
-    };
-    if constexpr (M == 3) {
-        order(0, 1); order(0, 2); order(1, 2);
-    } else if constexpr (M == 4) {
-        order(0, 1); order(2, 3); order(0, 2); order(1, 3); order(1, 2);
-    } else {
-        static_assert(M == 5, "3 to 5 components");
-        order(0, 1); order(3, 4); order(2, 4); order(2, 3); order(0, 3); order(0, 2);
-        order(1, 4); order(1, 3); order(1, 2);
-    }
-}
-
 // Background test (§III.A) of the changed component at rank `rank` after
 // the update: it is in B (the shortest rank prefix summing past T) unless the
 // prefix before it already sums past T (prefix sums of non-negative weights
@@ -420,33 +397,36 @@ __device__ __forceinline__ int mixture_step(Comp<D> (&c)[M], const float (&x)[D]
     return mixture_update<M, D, kOptions, -1>(c, x, p, lanes, hit, d2s);
 }
 
-// ------------------------------------------------- mixture step, FP32 state
-// The same tick of one mixture straight on the planes in memory. A tick
+// ------------------------------------- mixture step on what a pixel needs
+// The same tick of one mixture without the whole state in hand. A tick
 // changes every weight, and of the means and variances only those of the
 // component that matched or was replaced, unless components change places.
 // So it needs every weight and variance (the ranking) and the best-ranked
-// component's mean, loaded by the caller; the other means are loaded only in
-// lanes that do not match the best-ranked component or whose components
-// change places, and only what changed is stored: of 16 M values moved per
-// pixel, 6 M + 10 remain for a background pixel. (Per-lane predicates: a warp
-// moves the 32-byte sectors its lanes ask for. A lane that stores a mean or
-// a variance has loaded that element, so a partly stored sector is one the L2
-// already holds.) The means are never all held in registers: where components
-// change places each plane is permuted on its own. Measured against moving
-// the whole state (HBM-bound at 100% of the copy bandwidth): one 1920x1080
-// camera, M = 5, 101.1 -> 70.1 us per tick (DRAM reads 108 instead of 165
-// bytes per pixel); 64 pooled cameras 2299 -> 1393 us.
+// component's mean, which the caller has loaded; the other means are loaded
+// only in lanes that do not match the best-ranked component or whose
+// components change places, and only what changed is stored: of 16 M values
+// moved per pixel, 6 M + 10 remain for a background pixel. (Per-lane
+// predicates: a warp moves the 32-byte sectors its lanes ask for. A lane that
+// stores a mean or a variance has loaded that element, so a partly stored
+// sector is one the L2 already holds.) Measured in FP32 against moving the
+// whole state (HBM-bound at 100% of the copy bandwidth): one 1920x1080
+// camera, M = 5, 101.1 -> 63.5 us per tick (DRAM reads 108 instead of 165
+// bytes per pixel); 64 pooled cameras 2299 -> 1369 us. (Re-reading means
+// where components change places, one plane at a time to save registers,
+// measured 70.1 and 1390 us.)
 //
-// at(i, k): reference to value k of component i, k = 0 the weight, 1..D the
-// mean, D + 1 the variance. w, v: the weights and variances; mu: the
-// best-ranked component's mean. kJ = 0: every lane of the call matched the
-// best-ranked component.
-template <int M, int D, bool kOptions, int kJ, class At>
-__device__ __forceinline__ int plane_update(At at, float (&w)[M], const float (&v)[M],
-                                            float (&mu)[D], const float (&x)[D],
-                                            const StreamPrm &p, uint32_t lanes, bool matched,
-                                            int j, float d2j) {
-    const int jj = kJ == 0 ? 0 : j;
+// Io is where the state lives: load_means(m) fills the means m[1..] of this
+// lane; put(r, mu, v) takes the new mean and variance at rank r
+// (r known at compile time, only for ranks that changed). w, v: the weights
+// (updated to the new ones, in rank order) and variances; mu: the best-ranked
+// component's mean.
+template <int M, int D, bool kOptions, int kJ, class Io>
+__device__ __forceinline__ int ranked_update(Io &io, float (&w)[M], const float (&v)[M],
+                                             float (&mu)[D], float (&m)[M][D],
+                                             const float (&x)[D], const StreamPrm &p,
+                                             uint32_t lanes, bool best, bool matched, int j,
+                                             float d2j) {
+    const int jj = kJ == 0 ? 0 : j; // the component that changes
     float vj = v[0];
     if (kJ != 0) {
 #pragma unroll
@@ -454,7 +434,9 @@ __device__ __forceinline__ int plane_update(At at, float (&w)[M], const float (&
             if (i == jj)
                 vj = v[i];
     }
-    // Weights: as in mixture_update.
+    // Weights decay; the matched one gains alpha, or the last-ranked one is
+    // replaced on a miss; then renormalise. (Explicitly rounded operations:
+    // no multiply-add contraction, so every path rounds alike.)
     float sum = 0.f;
 #pragma unroll
     for (int i = 0; i < M; ++i) {
@@ -465,6 +447,8 @@ __device__ __forceinline__ int plane_update(At at, float (&w)[M], const float (&
         sum = __fadd_rn(sum, wi);
     }
     const float inv = __fdividef(1.0f, sum); // within 2 ulp; the sum is near 1
+    // Mean and variance of the changed component (the variance from the
+    // squared distance to the new mean).
     if (matched) {
         float orho = p.oma, rho = p.alpha;
         if (kOptions)
@@ -483,6 +467,10 @@ __device__ __forceinline__ int plane_update(At at, float (&w)[M], const float (&
             mu[ch] = x[ch];
         vj = p.init_var;
     }
+    // Re-rank by w / sigma (stable), then the background test. When every
+    // lane's components are already in non-increasing key order (the usual
+    // case), the stable network would leave them as they are, so the warp
+    // skips it and the changed component keeps its rank.
     uint32_t key[M];
     bool sorted = true;
 #pragma unroll
@@ -492,48 +480,49 @@ __device__ __forceinline__ int plane_update(At at, float (&w)[M], const float (&
         if (i > 0)
             sorted = sorted && !(key[i] > key[i - 1]);
     }
-    int rank = jj;
+    int rank = jj; // the changed component's rank after the update
     if (__any_sync(lanes, !sorted)) {
-        // Sort (key, weight); the key's low bits say which component a rank
-        // holds (lanes that are in order keep theirs).
-        rank_sort<M>(key, w);
-        int id[M];
+        if (!sorted && (kJ == 0 || best))
+            io.load_means(m);
+        Comp<D> c[M];
 #pragma unroll
-        for (int r = 0; r < M; ++r) {
-            id[r] = 7 - (int)(key[r] & 7u);
-            if (id[r] == jj)
-                rank = r;
+        for (int i = 0; i < M; ++i) {
+            c[i].key = key[i];
+            c[i].w = w[i];
+            c[i].v = i == jj ? vj : v[i];
+#pragma unroll
+            for (int ch = 0; ch < D; ++ch)
+                c[i].mu[ch] = i == jj ? mu[ch] : m[i][ch];
         }
+        rank_sort<M, D>(c);
 #pragma unroll
-        for (int k = 1; k <= D + 1; ++k) {
-            float val[M];
-#pragma unroll
-            for (int r = 0; r < M; ++r) {
-                val[r] = k <= D ? mu[k <= D ? k - 1 : 0] : vj;
-                if (id[r] != r && id[r] != jj)
-                    val[r] = at(id[r], k);
-            }
-#pragma unroll
-            for (int r = 0; r < M; ++r)
-                if (id[r] != r || id[r] == jj)
-                    at(r, k) = val[r];
+        for (int r = 0; r < M; ++r) { // the stored rank is in the key
+            const int id = 7 - (int)(c[r].key & 7u);
+            if (id == jj)
+                rank = r;
+            w[r] = c[r].w;
+            if (id == jj || id != r)
+                io.put(r, c[r].mu, c[r].v);
         }
     } else {
 #pragma unroll
-        for (int ch = 0; ch < D; ++ch)
-            at(jj, 1 + ch) = mu[ch];
-        at(jj, D + 1) = vj;
+        for (int r = 0; r < M; ++r)
+            if (r == jj)
+                io.put(r, mu, vj);
     }
-#pragma unroll
-    for (int r = 0; r < M; ++r)
-        at(r, 0) = w[r];
     return background_test<M>(w, rank, matched, p.T);
 }
 
-template <int M, int D, bool kOptions, class At>
-__device__ __forceinline__ int plane_step(At at, float (&w)[M], const float (&v)[M],
-                                          float (&mu)[D], const float (&x)[D],
-                                          const StreamPrm &p, uint32_t lanes) {
+// One tick of one mixture at one pixel (§III.A). The components are in rank
+// order on entry and on exit. Returns the stream's foreground bit. lanes: the
+// set of lanes of the warp that make this same call, computed by the caller
+// before the code diverged. Two paths, which compute the same: one
+// specialised to a match of the best-ranked component in every lane of the
+// call (the usual case for background pixels), and the general one.
+template <int M, int D, bool kOptions, class Io>
+__device__ __forceinline__ int ranked_step(Io &io, float (&w)[M], const float (&v)[M],
+                                           float (&mu)[D], const float (&x)[D],
+                                           const StreamPrm &p, uint32_t lanes) {
     float d2 = 0.f;
 #pragma unroll
     for (int ch = 0; ch < D; ++ch) {
@@ -541,35 +530,36 @@ __device__ __forceinline__ int plane_step(At at, float (&w)[M], const float (&v)
         d2 = fmaf(df, df, d2);
     }
     const bool best = d2 < p.k2 * v[0];
+    float m[M][D] = {};
     if (__all_sync(lanes, best))
-        return plane_update<M, D, kOptions, 0>(at, w, v, mu, x, p, lanes, true, 0, d2);
+        return ranked_update<M, D, kOptions, 0>(io, w, v, mu, m, x, p, lanes, true, true, 0, d2);
     bool matched = best;
     int jj = 0;
-    if (!best) {
+    if (!best) { // the first match, in rank order, within k standard deviations
         jj = M - 1; // replaced on a miss
-        float d2s[M];
-#pragma unroll
-        for (int i = 1; i < M; ++i) {
-            d2s[i] = 0.f;
-#pragma unroll
-            for (int ch = 0; ch < D; ++ch) {
-                const float df = x[ch] - at(i, 1 + ch);
-                d2s[i] = fmaf(df, df, d2s[i]);
-            }
-        }
-#pragma unroll
-        for (int i = M - 1; i >= 1; --i) { // the first match wins
-            if (d2s[i] < p.k2 * v[i]) {
-                matched = true;
-                jj = i;
-                d2 = d2s[i];
-            }
-        }
+        io.load_means(m);
 #pragma unroll
         for (int ch = 0; ch < D; ++ch)
-            mu[ch] = at(jj, 1 + ch);
+            m[0][ch] = mu[ch];
+#pragma unroll
+        for (int i = M - 1; i >= 1; --i) {
+            float d2i = 0.f;
+#pragma unroll
+            for (int ch = 0; ch < D; ++ch) {
+                const float df = x[ch] - m[i][ch];
+                d2i = fmaf(df, df, d2i);
+            }
+            if (d2i < p.k2 * v[i]) {
+                matched = true;
+                jj = i;
+                d2 = d2i;
+#pragma unroll
+                for (int ch = 0; ch < D; ++ch)
+                    mu[ch] = m[i][ch];
+            }
+        }
     }
-    return plane_update<M, D, kOptions, -1>(at, w, v, mu, x, p, lanes, matched, jj, d2);
+    return ranked_update<M, D, kOptions, -1>(io, w, v, mu, m, x, p, lanes, best, matched, jj, d2);
 }
 
 // List 1 (§III.C) on the low four bits of the per-pixel byte.
@@ -630,6 +620,28 @@ __device__ __forceinline__ void first_pixel_f32(const CamView &cv, int64_t p, in
                                  : (uint8_t)fuse_list1(0, 0, depth ? kDepthStarted : 0u);
 }
 
+// Planes of one pixel's FP32 state as ranked_step's Io: D mean planes from
+// field kMu, the variance plane kV. (D = 4: the fourth mean is the depth's.)
+template <int M, int D, int kMu, int kV> struct PlanesF32 {
+    float *b;
+    static __device__ __forceinline__ constexpr int mean(int ch) {
+        return ch < 3 ? kMu + ch : F_MUD;
+    }
+    __device__ __forceinline__ void load_means(float (&m)[M][D]) const {
+#pragma unroll
+        for (int i = 1; i < M; ++i)
+#pragma unroll
+            for (int ch = 0; ch < D; ++ch)
+                m[i][ch] = b[(kFields * i + mean(ch)) * kTile];
+    }
+    __device__ __forceinline__ void put(int r, const float (&mu)[D], float v) const {
+#pragma unroll
+        for (int ch = 0; ch < D; ++ch)
+            b[(kFields * r + mean(ch)) * kTile] = mu[ch];
+        b[(kFields * r + kV) * kTile] = v;
+    }
+};
+
 // FP32 state after the first tick. The loads that every lane needs come
 // first, for both mixtures together.
 template <int M, int kVariant>
@@ -637,44 +649,40 @@ __device__ __forceinline__ uint32_t tick_pixel_f32(const CamView &cv, int64_t p,
                                                    const float (&xc)[3], uint32_t draw,
                                                    uint32_t lanes_c) {
     float *const b = static_cast<float *>(cv.planes) + e0;
+    auto at = [b](int i, int f) -> float & { return b[(kFields * i + f) * kTile]; };
     float w[M], v[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        w[i] = at(i, F_WC);
+        v[i] = at(i, F_VC);
+    }
     if constexpr (kVariant == 2) {
         // The augmentation alternative (§III.B): one mixture over R, G, B and
         // the scaled depth, stored in the colour planes plus the depth-mean
         // plane. A zero reading takes the best-ranked component's depth mean.
-        auto at = [b](int i, int k) -> float & {
-            const int f = k < 4 ? F_WC + k : k == 4 ? F_MUD : F_VC;
-            return b[(kFields * i + f) * kTile];
-        };
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-            w[i] = at(i, 0);
-            v[i] = at(i, 5);
-        }
-        float mu[4] = {at(0, 1), at(0, 2), at(0, 3), at(0, 4)};
+        float mu[4] = {at(0, F_MUR), at(0, F_MUG), at(0, F_MUB), at(0, F_MUD)};
         const float xa[4] = {xc[0], xc[1], xc[2], draw ? cv.depth_scale * (float)draw : mu[3]};
-        const uint32_t f = (uint32_t)plane_step<M, 4, true>(at, w, v, mu, xa, cv.pc, lanes_c);
+        PlanesF32<M, 4, F_MUR, F_VC> io = {b};
+        const uint32_t f = (uint32_t)ranked_step<M, 4, true>(io, w, v, mu, xa, cv.pc, lanes_c);
+#pragma unroll
+        for (int r = 0; r < M; ++r)
+            at(r, F_WC) = w[r];
         cv.fusion[p] = (uint8_t)f;
         return f | (f << 1) | (f << 2);
     } else {
-        auto at_c = [b](int i, int k) -> float & {
-            return b[(kFields * i + F_WC + k) * kTile];
-        };
-        auto at_d = [b](int i, int k) -> float & {
-            return b[(kFields * i + F_WD + k) * kTile];
-        };
-        float wd[M], vd[M];
         const uint32_t fb0 = cv.fusion[p];
+        float mu[3] = {at(0, F_MUR), at(0, F_MUG), at(0, F_MUB)};
+        float wd[M], vd[M], mud[1] = {at(0, F_MUD)};
 #pragma unroll
         for (int i = 0; i < M; ++i) {
-            w[i] = at_c(i, 0);
-            v[i] = at_c(i, 4);
-            wd[i] = at_d(i, 0);
-            vd[i] = at_d(i, 2);
+            wd[i] = at(i, F_WD);
+            vd[i] = at(i, F_VD);
         }
-        float mu[3] = {at_c(0, 1), at_c(0, 2), at_c(0, 3)};
-        float mud[1] = {at_d(0, 1)};
-        const int fgc = plane_step<M, 3, (kVariant != 0)>(at_c, w, v, mu, xc, cv.pc, lanes_c);
+        PlanesF32<M, 3, F_MUR, F_VC> colour = {b};
+        const int fgc = ranked_step<M, 3, (kVariant != 0)>(colour, w, v, mu, xc, cv.pc, lanes_c);
+#pragma unroll
+        for (int r = 0; r < M; ++r)
+            at(r, F_WC) = w[r];
         // The lanes that run the depth mixture: a reading, and a started model.
         uint32_t fb = fb0;
         const uint32_t lanes_d = __ballot_sync(lanes_c, draw != 0u && (fb & kDepthStarted));
@@ -684,15 +692,19 @@ __device__ __forceinline__ uint32_t tick_pixel_f32(const CamView &cv, int64_t p,
         } else if (!(fb & kDepthStarted)) {
 #pragma unroll
             for (int i = 0; i < M; ++i) {
-                at_d(i, 0) = 1.0f / (float)M;
-                at_d(i, 1) = (float)draw;
-                at_d(i, 2) = cv.pd.init_var;
+                at(i, F_WD) = 1.0f / (float)M;
+                at(i, F_MUD) = (float)draw;
+                at(i, F_VD) = cv.pd.init_var;
             }
             fb |= kDepthStarted;
             fgd = 0;
         } else {
             const float xd[1] = {(float)draw};
-            fgd = plane_step<M, 1, (kVariant != 0)>(at_d, wd, vd, mud, xd, cv.pd, lanes_d);
+            PlanesF32<M, 1, F_MUD, F_VD> depth = {b};
+            fgd = ranked_step<M, 1, (kVariant != 0)>(depth, wd, vd, mud, xd, cv.pd, lanes_d);
+#pragma unroll
+            for (int r = 0; r < M; ++r)
+                at(r, F_WD) = wd[r];
         }
         fb = fuse_list1(fgc, fgd, fb);
         if (fb != fb0)

@@ -4,7 +4,7 @@
 //
 // The tick is a stream over the mixture state: per pixel FP32 state needs
 // about 24 M + 40 bytes of it (what a tick reads and changes, see
-// plane_update), FP16/BF16 state moves all 32 M; plus 5 bytes of frame, the
+// ranked_update), FP16/BF16 state moves all 32 M; plus 5 bytes of frame, the
 // List-1 byte and 1/8 byte of mask. There is no dense contraction, so there
 // is no tensor-core work; the design goal is full-line coalesced traffic
 // with enough bytes in flight per SM.
@@ -65,9 +65,9 @@ __device__ __forceinline__ void tick_body2(const CamView &cv) {
             write_mask_words(cv, (base >> 5) + u, bits[u]);
 }
 
-// FP32 state: latency-bound (64 registers and 32 warps per SM at M = 5; bounds
-// of 48 and 40 registers measured 66 and 70 us against 70 at 1920x1080, but
-// slower for M = 3). FP16/BF16 state: issue bound; at least 1024 threads per SM. V: process_pixel's variant (the options are separate
+// FP32 state: 64 registers and 32 warps per SM at M = 5; 5.9 of the 6.3 TB/s
+// that this mix of reads and partial writes reaches in the pooled kernel, the
+// rest being each launch's ramp and drain (about 7 us). FP16/BF16 state: issue bound; at least 1024 threads per SM. V: process_pixel's variant (the options are separate
 // instantiations, so the default kernels carry none of them). Small CTAs
 // measured faster than 256 threads: a CTA's slot frees as soon as its own
 // warps finish. A persistent grid-stride form measured slower (its loop
