@@ -216,7 +216,7 @@ void float_to_plane(const float *src, int elem, bool weight, int stride, int slo
 
 // Where one plane lives: in every tile, a run of `run` bytes starting `off`
 // bytes into the tile, holding its value of tile pixel t at element
-// t * stride + slot (FP32: the plane itself; FP16/BF16: its group).
+// t * stride + slot (FP32: the plane itself; FP16/BF16: its plane of pairs).
 struct PlaneRun {
     size_t off, run;
     int stride, slot;
@@ -225,14 +225,14 @@ PlaneRun plane_run(const Layout &L, int comp, int plane) {
     PlaneRun r;
     if (L.elem == 4) {
         r.run = (size_t)gmmdev::kTile * 4;
-        r.off = (size_t)gmmdev::tile_elem<0>(comp, plane, 0) * 4;
+        r.off = (size_t)(gmmdev::kFields * comp + plane) * gmmdev::kTile * 4;
         r.stride = 1;
         r.slot = 0;
     } else {
-        r.run = (size_t)gmmdev::kTile * 8;
-        r.off = (size_t)gmmdev::tile_elem<1>(comp, plane, 0) / 4 * 8;
-        r.stride = 4;
-        r.slot = gmmdev::h16_slot(plane);
+        r.run = (size_t)gmmdev::kTile * 4;
+        r.off = (size_t)gmmdev::pair_plane(L.planes_per_tile / gmmdev::kFields, comp, plane) * r.run;
+        r.stride = 2;
+        r.slot = gmmdev::pair_slot(plane);
     }
     return r;
 }
@@ -262,7 +262,7 @@ int state_get_common(const gmm_config &c, const Layout &L, const void *arena,
         return GMM_OK;
     }
     const bool weight = plane == GMM_PLANE_W_C || plane == GMM_PLANE_W_D;
-    // The plane (or its group) is a run of bytes in every tile: a pitched copy.
+    // The plane (or its pairs) is a run of bytes in every tile: a pitched copy.
     const PlaneRun r = plane_run(L, comp, plane);
     std::vector<uint8_t> tmp((size_t)L.n_tiles * r.run);
     const uint8_t *src = static_cast<const uint8_t *>(arena) + r.off;
@@ -305,7 +305,7 @@ int state_set_common(const gmm_config &c, const Layout &L, void *arena, cudaStre
         std::vector<uint8_t> tmp((size_t)L.n_tiles * r.run, 0);
         uint8_t *dst = static_cast<uint8_t *>(arena) + r.off;
         e = cudaSuccess;
-        if (r.stride > 1) // the group's other slots keep their values
+        if (r.stride > 1) // the pairs' other slots keep their values
             e = cudaMemcpy2DAsync(tmp.data(), r.run, dst, L.tile_bytes, r.run,
                                   (size_t)L.n_tiles, cudaMemcpyDeviceToHost, stream);
         if (e == cudaSuccess)

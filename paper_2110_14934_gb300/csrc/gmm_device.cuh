@@ -12,11 +12,17 @@
 //   FP32: one plane per field, element (8 i + field) * kTile + t for tile
 //         pixel t: a warp reads 32 consecutive floats of a plane, one fully
 //         used 128-byte line;
-//   FP16/BF16: two groups of four 2-byte slots per component and pixel,
-//         group 0 = {w_c, w_d, mu_r, mu_g}, group 1 = {mu_b, v_c, mu_d, v_d},
-//         element ((2 i + group) * kTile + t) * 4 + slot: one 8-byte access
-//         moves a group (a warp: 256 contiguous bytes), and each 4-byte half
-//         holds two values of one type, converted by one packed instruction.
+//   FP16/BF16: planes of 4-byte pairs of one type, element (plane * kTile +
+//         t) * 2 + slot: W_i = {w_c, w_d} at plane 2 i, V_i = {v_c, v_d} at
+//         2 i + 1, RG_i = {mu_r, mu_g} at 2 M + 2 i, BD_i = {mu_b, mu_d} at
+//         2 M + 2 i + 1: what every tick reads (all W and V, RG_0, BD_0) is
+//         one contiguous block at the head of the tile, the other means
+//         follow; a warp's access is one fully used 128-byte line, converted
+//         by one packed instruction per pixel;
+//   FP16/BF16 state that the caller owns (documented in gmm.h): two groups
+//         of four 2-byte slots per component and pixel, group 0 = {w_c, w_d,
+//         mu_r, mu_g}, group 1 = {mu_b, v_c, mu_d, v_d}, element ((2 i +
+//         group) * kTile + t) * 4 + slot.
 // The offsets of a pixel's values are compile-time constants from one base
 // address, and a tile's whole state is one contiguous block that a single
 // bulk copy moves. The List-1 byte of a pixel lives in a separate byte array
@@ -26,6 +32,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 namespace gmmdev {
 
@@ -39,18 +47,17 @@ constexpr int kStochasticWeights = 4; // CamView.flags: BF16 weights stored with
 constexpr uint32_t kRhoEta = 1u;        // StreamPrm.flags: rho = alpha * eta(x | mu, sigma)
 constexpr uint32_t kVarPerChannel = 2u; // StreamPrm.flags: v is the per-channel variance
 
-// Group and slot of a field in the FP16/BF16 layout.
-__host__ __device__ constexpr int h16_group(int f) {
-    return (f == F_MUB || f == F_VC || f == F_MUD || f == F_VD) ? 1 : 0;
+// Storage of the state, as the kernels' PREC (CamView.prec).
+enum { kF32 = 0, kF16 = 1, kF16Caller = 2 };
+
+// Plane and slot of a field of component i in the FP16/BF16 pair layout.
+__host__ __device__ constexpr int pair_plane(int M, int i, int f) {
+    return f == F_WC || f == F_WD ? 2 * i
+         : f == F_VC || f == F_VD ? 2 * i + 1
+         : f == F_MUR || f == F_MUG ? 2 * M + 2 * i : 2 * M + 2 * i + 1;
 }
-__host__ __device__ constexpr int h16_slot(int f) {
-    return (f == F_WC || f == F_MUB) ? 0 : (f == F_WD || f == F_VC) ? 1
-                                     : (f == F_MUR || f == F_MUD) ? 2 : 3;
-}
-// Element index, within its tile, of field f of component i at tile pixel t.
-template <int PREC> __host__ __device__ constexpr int tile_elem(int i, int f, int t) {
-    return PREC == 0 ? (kFields * i + f) * kTile + t
-                     : ((2 * i + h16_group(f)) * kTile + t) * 4 + h16_slot(f);
+__host__ __device__ constexpr int pair_slot(int f) {
+    return f == F_WD || f == F_VD || f == F_MUG || f == F_MUD ? 1 : 0;
 }
 
 struct StreamPrm {
@@ -103,7 +110,7 @@ struct CamView {
     int64_t n_tiles;       // state tiles: ceil(n_pad / kTile)
     int64_t n_pad;         // H*w_pad (< 2^30)
     int H, W, w_pad, wpr;  // wpr = words per mask row = w_pad / 32
-    int M, prec, first, flags; // flags: kStageInputs, kModeAugmented, kStochasticWeights
+    int M, prec, first, flags; // prec: kF32..; flags: kStageInputs, kModeAugmented, kStochasticWeights
     uint32_t wpr_mul, wpr_shift; // n / wpr == umulhi(n, wpr_mul) >> wpr_shift (wpr > 1)
     float depth_scale;           // augmented mode: depth (mm) to the colour byte range
     uint32_t tick;               // ticks the model has taken (seeds stochastic rounding)
@@ -163,21 +170,12 @@ __device__ __forceinline__ uint32_t bf16x2_pack_sr(float lo, float hi, uint32_t 
     return h | l;
 }
 
-// The eight values of one component at one pixel.
-struct Fields {
-    float wc, mur, mug, mub, vc, wd, mud, vd;
-};
-
-// Store component i (FP16/BF16 state) of the pixel in column t of the tile
-// that starts at element tb. sr: nonzero = 32 random bits for the stochastic
-// rounding of the two weights (kSR builds only).
-template <bool kSR>
-__device__ __forceinline__ void store_fields_f16(void *pl, int64_t tb, uint32_t t, int i,
-                                                 const Fields &f, uint32_t sr) {
-    uint2 *g = static_cast<uint2 *>(pl) + (tb >> 2) + t + 2 * i * kTile;
-    const uint32_t w = (kSR && sr) ? bf16x2_pack_sr(f.wc, f.wd, sr) : bf16x2_pack(f.wc, f.wd);
-    g[0] = make_uint2(w, f16x2_pack_sat(f.mur, f.mug));
-    g[kTile] = make_uint2(f16x2_pack_sat(f.mub, f.vc), f16x2_pack_sat(f.mud, f.vd));
+// Replace the low / high half of a pair, rounded like f16x2_pack_sat.
+__device__ __forceinline__ uint32_t f16x2_set_lo(uint32_t pair, float lo) {
+    return __byte_perm(f16x2_pack_sat(lo, lo), pair, 0x7610);
+}
+__device__ __forceinline__ uint32_t f16x2_set_hi(uint32_t pair, float hi) {
+    return __byte_perm(f16x2_pack_sat(hi, hi), pair, 0x1054);
 }
 
 // ------------------------------------------------------------ mixture step
@@ -252,154 +250,7 @@ __device__ __forceinline__ int background_test(const float (&w)[M], int rank, bo
     }
     return (!matched || before > T) ? 1 : 0;
 }
-template <int M, int D>
-__device__ __forceinline__ int background_test(const Comp<D> (&c)[M], int rank, bool matched,
-                                               float T) {
-    float w[M];
-#pragma unroll
-    for (int r = 0; r < M; ++r)
-        w[r] = c[r].w;
-    return background_test<M>(w, rank, matched, T);
-}
-
-// The update after the match (§III.A): weights, the changed component's mean
-// and variance, re-ranking and the background test. hit: bit i set when
-// component i lies within k standard deviations (the first set bit is the
-// match); d2s: the squared distances. kJ >= 0: every lane of this call
-// matched component kJ (the changed component is then known at compile time
-// and needs no selects); kJ < 0: any outcome.
-template <int M, int D, bool kOptions, int kJ>
-__device__ __forceinline__ int mixture_update(Comp<D> (&c)[M], const float (&x)[D],
-                                              const StreamPrm &p, uint32_t lanes, uint32_t hit,
-                                              const float (&d2s)[M]) {
-    const bool matched = kJ >= 0 || hit != 0u;
-    const int jj = kJ >= 0 ? kJ : (matched ? __ffs(hit) - 1 : M - 1);
-    float d2j = d2s[0];
-    if (kOptions) {
-#pragma unroll
-        for (int i = 1; i < M; ++i)
-            if (i == jj)
-                d2j = d2s[i];
-    }
-
-    // The component that changes (matched, or the last-ranked on a miss),
-    // gathered once.
-    float muj[D], vj = c[0].v;
-#pragma unroll
-    for (int ch = 0; ch < D; ++ch)
-        muj[ch] = c[0].mu[ch];
-#pragma unroll
-    for (int i = 1; i < M; ++i) {
-        if (i == jj) {
-            vj = c[i].v;
-#pragma unroll
-            for (int ch = 0; ch < D; ++ch)
-                muj[ch] = c[i].mu[ch];
-        }
-    }
-
-    // Weights decay; the matched one gains alpha, or the last-ranked one is
-    // replaced on a miss; then renormalise. (Explicitly rounded operations:
-    // no multiply-add contraction, so every path rounds alike.)
-    float sum = 0.f;
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-        float w = __fmul_rn(c[i].w, p.oma);
-        if (i == jj)
-            w = matched ? __fadd_rn(w, p.alpha) : p.init_w;
-        c[i].w = w;
-        sum = __fadd_rn(sum, w);
-    }
-    const float inv = __fdividef(1.0f, sum); // within 2 ulp; the sum is near 1
-
-    // Mean and variance of the changed component (the variance from the
-    // squared distance to the new mean).
-    if (matched) {
-        float orho = p.oma, rho = p.alpha;
-        if (kOptions)
-            rho = match_rate<D>(p, d2j, vj, orho);
-        float d2n = 0.f;
-#pragma unroll
-        for (int ch = 0; ch < D; ++ch) {
-            muj[ch] = fmaf(orho, muj[ch], rho * x[ch]);
-            const float df = x[ch] - muj[ch];
-            d2n = fmaf(df, df, d2n);
-        }
-        vj = fmaxf(p.v_min, fmaf(orho, vj, rho * (kOptions ? var_sample<D>(p, d2n) : d2n)));
-    } else {
-#pragma unroll
-        for (int ch = 0; ch < D; ++ch)
-            muj[ch] = x[ch];
-        vj = p.init_var;
-    }
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-        c[i].w *= inv;
-        if (i == jj) {
-#pragma unroll
-            for (int ch = 0; ch < D; ++ch)
-                c[i].mu[ch] = muj[ch];
-            c[i].v = vj;
-        }
-        c[i].key = rank_key(c[i].w, c[i].v, i);
-    }
-
-    // Re-rank by w / sigma (stable), then the background test. When every
-    // lane's components are already in non-increasing key order (the usual
-    // case: a background pixel matches its best component and the others
-    // decay by the same factor), the stable network would leave them as they
-    // are, so the warp skips it and the changed component keeps its rank.
-    bool sorted = true;
-#pragma unroll
-    for (int i = 1; i < M; ++i)
-        sorted = sorted && !(c[i].key > c[i - 1].key);
-    int rank = jj; // the changed component's rank after the update
-    if (__any_sync(lanes, !sorted)) {
-        rank_sort<M, D>(c);
-#pragma unroll
-        for (int r = 0; r < M; ++r)
-            if ((c[r].key & 7u) == 7u - (uint32_t)jj) // its stored rank, from the key
-                rank = r;
-        if (kJ >= 0) // (the specialised path keeps its rank known where no sort ran)
-            return background_test<M, D>(c, rank, matched, p.T);
-    }
-    return background_test<M, D>(c, rank, matched, p.T);
-}
-
-// One tick of one mixture at one pixel (§III.A). The components are in rank
-// order on entry and on exit. Returns the stream's foreground bit. A warp
-// skips the sorting network when it would change nothing; `lanes` is the set
-// of lanes of the warp that make this same call, computed by the caller
-// before the code diverged. Where every lane of the call matches its
-// best-ranked component (the usual case for background pixels) a path
-// specialised to that runs; it computes exactly what the general path does.
-template <int M, int D, bool kOptions>
-__device__ __forceinline__ int mixture_step(Comp<D> (&c)[M], const float (&x)[D],
-                                            const StreamPrm &p, uint32_t lanes) {
-    // Match: first component, in rank order, within k standard deviations
-    // (bit i of hit: component i is within; the first set bit wins).
-    uint32_t hit = 0u;
-    float d2s[M];
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-        float d2 = 0.f;
-#pragma unroll
-        for (int ch = 0; ch < D; ++ch) {
-            const float df = x[ch] - c[i].mu[ch];
-            d2 = fmaf(df, df, d2);
-        }
-        d2s[i] = d2;
-        if (d2 < p.k2 * c[i].v)
-            hit |= 1u << i;
-    }
-    if (__all_sync(lanes, hit & 1u))
-        return mixture_update<M, D, kOptions, 0>(c, x, p, lanes, hit, d2s);
-    return mixture_update<M, D, kOptions, -1>(c, x, p, lanes, hit, d2s);
-}
-
-// ------------------------------------- mixture step on what a pixel needs
-// The same tick of one mixture without the whole state in hand. A tick
-// changes every weight, and of the means and variances only those of the
+// One tick of one mixture without the whole state in hand. A tick changes every weight, and of the means and variances only those of the
 // component that matched or was replaced, unless components change places.
 // So it needs every weight and variance (the ranking) and the best-ranked
 // component's mean, which the caller has loaded; the other means are loaded
@@ -410,63 +261,112 @@ __device__ __forceinline__ int mixture_step(Comp<D> (&c)[M], const float (&x)[D]
 // stores a mean or a variance has loaded that element, so a partly stored
 // sector is one the L2 already holds.) Measured in FP32 against moving the
 // whole state (HBM-bound at 100% of the copy bandwidth): one 1920x1080
-// camera, M = 5, 101.1 -> 63.5 us per tick (DRAM reads 108 instead of 165
-// bytes per pixel); 64 pooled cameras 2299 -> 1369 us. (Re-reading means
-// where components change places, one plane at a time to save registers,
-// measured 70.1 and 1390 us.)
+// camera, M = 5, 101.1 -> 64.7 us per tick (DRAM reads 108 instead of 165
+// bytes per pixel); 64 pooled cameras 2299 -> 1371 us. In FP16/BF16: 54.7 ->
+// 45.7 us, with the caller's layout (whose weights share a group with means)
+// 1280x720, M = 4, with opening 25.5 -> 23.3 us.
 //
-// Io is where the state lives: load_means(m) fills the means m[1..] of this
-// lane; put(r, mu, v) takes the new mean and variance at rank r
+// Io is where the state lives: load_means(m, i0) fills this lane's stored
+// means m[i0..]; put(r, mu, v) takes the new mean and variance at rank r
 // (r known at compile time, only for ranks that changed). w, v: the weights
 // (updated to the new ones, in rank order) and variances; mu: the best-ranked
 // component's mean.
-template <int M, int D, bool kOptions, int kJ, class Io>
-__device__ __forceinline__ int ranked_update(Io &io, float (&w)[M], const float (&v)[M],
-                                             float (&mu)[D], float (&m)[M][D],
-                                             const float (&x)[D], const StreamPrm &p,
-                                             uint32_t lanes, bool best, bool matched, int j,
-                                             float d2j) {
-    const int jj = kJ == 0 ? 0 : j; // the component that changes
-    float vj = v[0];
-    if (kJ != 0) {
+// Returns the stream's foreground bit. lanes: the set of lanes of the warp that
+// make this same call, computed by the caller before the code diverged. Where
+// every lane of the call matches its best-ranked component (the usual case
+// for background pixels) the update is specialised to that; it computes
+// exactly what the general one does. The ranking is one copy of code for both,
+// and means are read again where components change places: with a ranking
+// per path the pooled FP16/BF16 kernel, which holds a body per M, spent a
+// third of its time on instruction fetch (24 cameras of odd sizes: 495 us
+// against 404; FP32 1920x1080 63.5 against 64.7).
+template <int D, bool kOptions>
+__device__ __forceinline__ float moved_component(float (&mu)[D], float v, const float (&x)[D],
+                                                 const StreamPrm &p, float d2) {
+    float orho = p.oma, rho = p.alpha;
+    if (kOptions)
+        rho = match_rate<D>(p, d2, v, orho);
+    float d2n = 0.f; // the variance follows the squared distance to the new mean
 #pragma unroll
-        for (int i = 1; i < M; ++i)
-            if (i == jj)
-                vj = v[i];
+    for (int ch = 0; ch < D; ++ch) {
+        mu[ch] = fmaf(orho, mu[ch], rho * x[ch]);
+        const float df = x[ch] - mu[ch];
+        d2n = fmaf(df, df, d2n);
     }
-    // Weights decay; the matched one gains alpha, or the last-ranked one is
-    // replaced on a miss; then renormalise. (Explicitly rounded operations:
-    // no multiply-add contraction, so every path rounds alike.)
-    float sum = 0.f;
+    return fmaxf(p.v_min, fmaf(orho, v, rho * (kOptions ? var_sample<D>(p, d2n) : d2n)));
+}
+
+template <int M, int D, bool kOptions, class Io>
+__device__ __forceinline__ int ranked_step(Io &io, float (&w)[M], float (&v)[M], float (&mu)[D],
+                                           const float (&x)[D], const StreamPrm &p,
+                                           uint32_t lanes) {
+    float d2 = 0.f;
 #pragma unroll
-    for (int i = 0; i < M; ++i) {
-        float wi = __fmul_rn(w[i], p.oma);
-        if (i == jj)
-            wi = matched ? __fadd_rn(wi, p.alpha) : p.init_w;
-        w[i] = wi;
-        sum = __fadd_rn(sum, wi);
+    for (int ch = 0; ch < D; ++ch) {
+        const float df = x[ch] - mu[ch];
+        d2 = fmaf(df, df, d2);
+    }
+    const bool best = d2 < p.k2 * v[0];
+    const bool all_best = __all_sync(lanes, best);
+    bool matched = best;
+    int jj = 0; // the component that changes
+    float sum;
+    // Weights decay; the matched one gains alpha, or the last-ranked one is
+    // replaced on a miss; then (below) renormalise. (Explicitly rounded
+    // operations: no multiply-add contraction, so both paths round alike.)
+    if (all_best) {
+        w[0] = sum = __fadd_rn(__fmul_rn(w[0], p.oma), p.alpha);
+#pragma unroll
+        for (int i = 1; i < M; ++i) {
+            w[i] = __fmul_rn(w[i], p.oma);
+            sum = __fadd_rn(sum, w[i]);
+        }
+        v[0] = moved_component<D, kOptions>(mu, v[0], x, p, d2);
+    } else {
+        float vj = v[0];
+        if (!best) { // the first match, in rank order, within k standard deviations
+            jj = M - 1; // replaced on a miss
+            float m[M][D];
+            io.load_means(m, 1);
+#pragma unroll
+            for (int i = M - 1; i >= 1; --i) {
+                float d2i = 0.f;
+#pragma unroll
+                for (int ch = 0; ch < D; ++ch) {
+                    const float df = x[ch] - m[i][ch];
+                    d2i = fmaf(df, df, d2i);
+                }
+                if (d2i < p.k2 * v[i]) {
+                    matched = true;
+                    jj = i;
+                    d2 = d2i;
+                    vj = v[i];
+#pragma unroll
+                    for (int ch = 0; ch < D; ++ch)
+                        mu[ch] = m[i][ch];
+                }
+            }
+        }
+        if (matched) {
+            vj = moved_component<D, kOptions>(mu, vj, x, p, d2);
+        } else {
+#pragma unroll
+            for (int ch = 0; ch < D; ++ch)
+                mu[ch] = x[ch];
+            vj = p.init_var;
+        }
+        sum = 0.f;
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            w[i] = __fmul_rn(w[i], p.oma);
+            if (i == jj) {
+                w[i] = matched ? __fadd_rn(w[i], p.alpha) : p.init_w;
+                v[i] = vj;
+            }
+            sum = __fadd_rn(sum, w[i]);
+        }
     }
     const float inv = __fdividef(1.0f, sum); // within 2 ulp; the sum is near 1
-    // Mean and variance of the changed component (the variance from the
-    // squared distance to the new mean).
-    if (matched) {
-        float orho = p.oma, rho = p.alpha;
-        if (kOptions)
-            rho = match_rate<D>(p, d2j, vj, orho);
-        float d2n = 0.f;
-#pragma unroll
-        for (int ch = 0; ch < D; ++ch) {
-            mu[ch] = fmaf(orho, mu[ch], rho * x[ch]);
-            const float df = x[ch] - mu[ch];
-            d2n = fmaf(df, df, d2n);
-        }
-        vj = fmaxf(p.v_min, fmaf(orho, vj, rho * (kOptions ? var_sample<D>(p, d2n) : d2n)));
-    } else {
-#pragma unroll
-        for (int ch = 0; ch < D; ++ch)
-            mu[ch] = x[ch];
-        vj = p.init_var;
-    }
     // Re-rank by w / sigma (stable), then the background test. When every
     // lane's components are already in non-increasing key order (the usual
     // case), the stable network would leave them as they are, so the warp
@@ -476,20 +376,21 @@ __device__ __forceinline__ int ranked_update(Io &io, float (&w)[M], const float 
 #pragma unroll
     for (int i = 0; i < M; ++i) {
         w[i] *= inv;
-        key[i] = rank_key(w[i], i == jj ? vj : v[i], i);
+        key[i] = rank_key(w[i], v[i], i);
         if (i > 0)
             sorted = sorted && !(key[i] > key[i - 1]);
     }
     int rank = jj; // the changed component's rank after the update
     if (__any_sync(lanes, !sorted)) {
-        if (!sorted && (kJ == 0 || best))
-            io.load_means(m);
+        float m[M][D] = {};
+        if (!sorted)
+            io.load_means(m, 0);
         Comp<D> c[M];
 #pragma unroll
         for (int i = 0; i < M; ++i) {
             c[i].key = key[i];
             c[i].w = w[i];
-            c[i].v = i == jj ? vj : v[i];
+            c[i].v = v[i];
 #pragma unroll
             for (int ch = 0; ch < D; ++ch)
                 c[i].mu[ch] = i == jj ? mu[ch] : m[i][ch];
@@ -504,62 +405,15 @@ __device__ __forceinline__ int ranked_update(Io &io, float (&w)[M], const float 
             if (id == jj || id != r)
                 io.put(r, c[r].mu, c[r].v);
         }
+    } else if (all_best) {
+        io.put(0, mu, v[0]);
     } else {
 #pragma unroll
         for (int r = 0; r < M; ++r)
             if (r == jj)
-                io.put(r, mu, vj);
+                io.put(r, mu, v[r]);
     }
     return background_test<M>(w, rank, matched, p.T);
-}
-
-// One tick of one mixture at one pixel (§III.A). The components are in rank
-// order on entry and on exit. Returns the stream's foreground bit. lanes: the
-// set of lanes of the warp that make this same call, computed by the caller
-// before the code diverged. Two paths, which compute the same: one
-// specialised to a match of the best-ranked component in every lane of the
-// call (the usual case for background pixels), and the general one.
-template <int M, int D, bool kOptions, class Io>
-__device__ __forceinline__ int ranked_step(Io &io, float (&w)[M], const float (&v)[M],
-                                           float (&mu)[D], const float (&x)[D],
-                                           const StreamPrm &p, uint32_t lanes) {
-    float d2 = 0.f;
-#pragma unroll
-    for (int ch = 0; ch < D; ++ch) {
-        const float df = x[ch] - mu[ch];
-        d2 = fmaf(df, df, d2);
-    }
-    const bool best = d2 < p.k2 * v[0];
-    float m[M][D] = {};
-    if (__all_sync(lanes, best))
-        return ranked_update<M, D, kOptions, 0>(io, w, v, mu, m, x, p, lanes, true, true, 0, d2);
-    bool matched = best;
-    int jj = 0;
-    if (!best) { // the first match, in rank order, within k standard deviations
-        jj = M - 1; // replaced on a miss
-        io.load_means(m);
-#pragma unroll
-        for (int ch = 0; ch < D; ++ch)
-            m[0][ch] = mu[ch];
-#pragma unroll
-        for (int i = M - 1; i >= 1; --i) {
-            float d2i = 0.f;
-#pragma unroll
-            for (int ch = 0; ch < D; ++ch) {
-                const float df = x[ch] - m[i][ch];
-                d2i = fmaf(df, df, d2i);
-            }
-            if (d2i < p.k2 * v[i]) {
-                matched = true;
-                jj = i;
-                d2 = d2i;
-#pragma unroll
-                for (int ch = 0; ch < D; ++ch)
-                    mu[ch] = m[i][ch];
-            }
-        }
-    }
-    return ranked_update<M, D, kOptions, -1>(io, w, v, mu, m, x, p, lanes, best, matched, jj, d2);
 }
 
 // List 1 (§III.C) on the low four bits of the per-pixel byte.
@@ -627,9 +481,9 @@ template <int M, int D, int kMu, int kV> struct PlanesF32 {
     static __device__ __forceinline__ constexpr int mean(int ch) {
         return ch < 3 ? kMu + ch : F_MUD;
     }
-    __device__ __forceinline__ void load_means(float (&m)[M][D]) const {
+    __device__ __forceinline__ void load_means(float (&m)[M][D], int i0) const {
 #pragma unroll
-        for (int i = 1; i < M; ++i)
+        for (int i = i0; i < M; ++i)
 #pragma unroll
             for (int ch = 0; ch < D; ++ch)
                 m[i][ch] = b[(kFields * i + mean(ch)) * kTile];
@@ -713,112 +567,280 @@ __device__ __forceinline__ uint32_t tick_pixel_f32(const CamView &cv, int64_t p,
     }
 }
 
-// FP16/BF16 state: every group is loaded, and written back.
-template <int M, int kVariant>
-__device__ __forceinline__ uint32_t tick_pixel_f16(const CamView &cv, int64_t p, int64_t tb,
-                                                   uint32_t t, const float (&xc)[3],
-                                                   uint32_t draw, uint32_t lanes_c) {
-    const float xd[1] = {(float)draw};
-    const uint2 *const g = static_cast<const uint2 *>(cv.planes) + (tb >> 2) + t;
-    auto store = [&](int i, const Fields &f) {
-        const uint32_t sr = kVariant != 0 ? sr_weights(cv, (uint32_t)p, i) : 0u;
-        store_fields_f16<kVariant != 0>(cv.planes, tb, t, i, f, sr);
-    };
-    if (kVariant == 2) {
-        Comp<4> a[M];
-        float xa[4] = {xc[0], xc[1], xc[2], cv.depth_scale * (float)draw};
-        int fg;
-        if (cv.first) {
-            if (draw == 0u)
-                xa[3] = 0.f;
+// One pixel's FP16/BF16 state in the pair layout. Values stay packed until
+// they are needed, and what did not change is never stored: the weights of
+// every component always are, V and BD where either mixture changed them.
+template <int M> struct PairsF16 {
+    uint32_t *b; // the pixel's element of the tile's first plane
+    uint32_t W[M], V[M], BD[M], RG0;
+    bool loaded = false; // BD[1..] hold the stored values (or newer ones)
+    uint32_t changed = 0u;
+
+    __device__ __forceinline__ PairsF16(void *planes, int64_t tile, uint32_t t)
+        : b(static_cast<uint32_t *>(planes) + tile * (4 * M * kTile) + t) {}
+    __device__ __forceinline__ uint32_t &at(int plane) const { return b[plane * kTile]; }
+    __device__ __forceinline__ void load() {
 #pragma unroll
-            for (int i = 0; i < M; ++i) {
-                a[i].w = 1.0f / (float)M;
-                a[i].mu[0] = xa[0]; a[i].mu[1] = xa[1]; a[i].mu[2] = xa[2]; a[i].mu[3] = xa[3];
-                a[i].v = cv.pc.init_var;
+        for (int i = 0; i < M; ++i) {
+            W[i] = at(2 * i);
+            V[i] = at(2 * i + 1);
+        }
+        RG0 = at(2 * M);
+        BD[0] = at(2 * M + 1);
+    }
+    __device__ __forceinline__ void load_bd() {
+        if (loaded)
+            return;
+        loaded = true;
+#pragma unroll
+        for (int i = 1; i < M; ++i)
+            BD[i] = at(2 * M + 2 * i + 1);
+    }
+    __device__ __forceinline__ float v_c(int i) const { return f16x2_unpack(V[i]).x; }
+    __device__ __forceinline__ float v_d(int i) const { return f16x2_unpack(V[i]).y; }
+    __device__ __forceinline__ float2 rg(int i) const {
+        return f16x2_unpack(i == 0 ? RG0 : at(2 * M + 2 * i));
+    }
+    __device__ __forceinline__ float mu_b(int i) const { return f16x2_unpack(BD[i]).x; }
+    __device__ __forceinline__ float mu_d(int i) const { return f16x2_unpack(BD[i]).y; }
+    __device__ __forceinline__ void load_c() { load_bd(); }
+    __device__ __forceinline__ void load_d() { load_bd(); }
+    __device__ __forceinline__ void put_c(int r, const float *mu, float v) {
+        at(2 * M + 2 * r) = f16x2_pack_sat(mu[0], mu[1]);
+        BD[r] = f16x2_set_lo(BD[r], mu[2]);
+        V[r] = f16x2_set_lo(V[r], v);
+        changed |= 1u << r;
+    }
+    __device__ __forceinline__ void put_d(int r, float mu, float v) {
+        BD[r] = f16x2_set_hi(BD[r], mu);
+        V[r] = f16x2_set_hi(V[r], v);
+        changed |= 1u << r;
+    }
+    __device__ __forceinline__ void clear_v_d() { // unused and read as zero (augmented mode)
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            if (V[i] >> 16) {
+                V[i] &= 0xffffu;
+                at(2 * i + 1) = V[i];
             }
-            fg = 0;
-        } else {
+        }
+    }
+    __device__ __forceinline__ void store(int i, uint32_t w) const {
+        at(2 * i) = w;
+        if (changed >> i & 1u) {
+            at(2 * i + 1) = V[i];
+            at(2 * M + 2 * i + 1) = BD[i];
+        }
+    }
+    // The first tick: component i whole.
+    __device__ __forceinline__ void store_all(int i, uint32_t w, const float *mu, float v_c,
+                                              float mu_d, float v_d) const {
+        at(2 * i) = w;
+        at(2 * i + 1) = f16x2_pack_sat(v_c, v_d);
+        at(2 * M + 2 * i) = f16x2_pack_sat(mu[0], mu[1]);
+        at(2 * M + 2 * i + 1) = f16x2_pack_sat(mu[2], mu_d);
+    }
+};
+
+// The same in the caller-owned layout: the first group of a component (it
+// holds the weights) is always stored, the second where it changed.
+template <int M> struct GroupsF16 {
+    uint2 *b;
+    uint32_t W[M], RG[M], BV[M], DV[M]; // {w_c, w_d}, {mu_r, mu_g}, {mu_b, v_c}, {mu_d, v_d}
+    uint32_t changed = 0u;
+
+    __device__ __forceinline__ GroupsF16(void *planes, int64_t tile, uint32_t t)
+        : b(static_cast<uint2 *>(planes) + tile * (2 * M * kTile) + t) {}
+    __device__ __forceinline__ void load() {
 #pragma unroll
-            for (int i = 0; i < M; ++i) {
-                const uint2 g0 = g[2 * i * kTile], g1 = g[(2 * i + 1) * kTile];
-                a[i].w = bf16_lo(g0.x);
-                const float2 rg = f16x2_unpack(g0.y), bv = f16x2_unpack(g1.x);
-                a[i].mu[0] = rg.x; a[i].mu[1] = rg.y; a[i].mu[2] = bv.x;
-                a[i].v = bv.y;
-                a[i].mu[3] = f16x2_unpack(g1.y).x;
+        for (int i = 0; i < M; ++i) {
+            const uint2 g0 = b[2 * i * kTile], g1 = b[(2 * i + 1) * kTile];
+            W[i] = g0.x;
+            RG[i] = g0.y;
+            BV[i] = g1.x;
+            DV[i] = g1.y;
+        }
+    }
+    __device__ __forceinline__ float v_c(int i) const { return f16x2_unpack(BV[i]).y; }
+    __device__ __forceinline__ float v_d(int i) const { return f16x2_unpack(DV[i]).y; }
+    __device__ __forceinline__ float2 rg(int i) const { return f16x2_unpack(RG[i]); }
+    __device__ __forceinline__ float mu_b(int i) const { return f16x2_unpack(BV[i]).x; }
+    __device__ __forceinline__ float mu_d(int i) const { return f16x2_unpack(DV[i]).x; }
+    __device__ __forceinline__ void load_c() {}
+    __device__ __forceinline__ void load_d() {}
+    __device__ __forceinline__ void load_bd() {}
+    __device__ __forceinline__ void put_c(int r, const float *mu, float v) {
+        RG[r] = f16x2_pack_sat(mu[0], mu[1]);
+        BV[r] = f16x2_pack_sat(mu[2], v);
+        changed |= 1u << r;
+    }
+    __device__ __forceinline__ void put_d(int r, float mu, float v) {
+        DV[r] = f16x2_pack_sat(mu, v);
+        changed |= 1u << r;
+    }
+    __device__ __forceinline__ void clear_v_d() {
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            if (DV[i] >> 16) {
+                DV[i] &= 0xffffu;
+                changed |= 1u << i;
             }
-            if (draw == 0u)
-                xa[3] = a[0].mu[3];
-            fg = mixture_step<M, 4, true>(a, xa, cv.pc, lanes_c);
-        }
-#pragma unroll
-        for (int i = 0; i < M; ++i) // w_d and v_d are unused and read as zero
-            store(i, {a[i].w, a[i].mu[0], a[i].mu[1], a[i].mu[2], a[i].v, 0.f, a[i].mu[3], 0.f});
-        const uint32_t f = (uint32_t)fg;
-        cv.fusion[p] = (uint8_t)f;
-        return f | (f << 1) | (f << 2);
-    }
-    Comp<3> c[M];
-    Comp<1> d[M];
-    uint32_t fb;
-    int fgc, fgd;
-    if (cv.first) {
-        fb = 0u;
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-            c[i].w = 1.0f / (float)M;
-            c[i].mu[0] = xc[0]; c[i].mu[1] = xc[1]; c[i].mu[2] = xc[2];
-            c[i].v = cv.pc.init_var;
-            d[i].w = 0.f; d[i].mu[0] = 0.f; d[i].v = 0.f;
-        }
-        fgc = 0;
-    } else {
-        // The depth values stay packed (two registers per component instead
-        // of three) while the colour mixture runs.
-        fb = cv.fusion[p];
-        uint32_t dw[M], dmv[M];
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-            const uint2 g0 = g[2 * i * kTile], g1 = g[(2 * i + 1) * kTile];
-            c[i].w = bf16_lo(g0.x);
-            const float2 rg = f16x2_unpack(g0.y), bv = f16x2_unpack(g1.x);
-            c[i].mu[0] = rg.x; c[i].mu[1] = rg.y; c[i].mu[2] = bv.x;
-            c[i].v = bv.y;
-            dw[i] = g0.x;
-            dmv[i] = g1.y;
-        }
-        fgc = mixture_step<M, 3, (kVariant != 0)>(c, xc, cv.pc, lanes_c);
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-            d[i].w = bf16_hi(dw[i]);
-            const float2 mv = f16x2_unpack(dmv[i]);
-            d[i].mu[0] = mv.x;
-            d[i].v = mv.y;
         }
     }
-    // The lanes that run the depth mixture: a reading, and a started model.
-    const uint32_t lanes_d = __ballot_sync(lanes_c, draw != 0u && (fb & kDepthStarted));
-    if (draw == 0u) {
-        fgd = fgc; // no reading: depth model untouched, depth answer = colour
-    } else if (!(fb & kDepthStarted)) {
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-            d[i].w = 1.0f / (float)M;
-            d[i].mu[0] = xd[0];
-            d[i].v = cv.pd.init_var;
-        }
-        fb |= kDepthStarted;
-        fgd = 0;
-    } else {
-        fgd = mixture_step<M, 1, (kVariant != 0)>(d, xd, cv.pd, lanes_d);
+    __device__ __forceinline__ void store(int i, uint32_t w) const {
+        b[2 * i * kTile] = make_uint2(w, RG[i]);
+        if (changed >> i & 1u)
+            b[(2 * i + 1) * kTile] = make_uint2(BV[i], DV[i]);
     }
-    fb = fuse_list1(fgc, fgd, fb);
+    __device__ __forceinline__ void store_all(int i, uint32_t w, const float *mu, float v_c,
+                                              float mu_d, float v_d) const {
+        b[2 * i * kTile] = make_uint2(w, f16x2_pack_sat(mu[0], mu[1]));
+        b[(2 * i + 1) * kTile] = make_uint2(f16x2_pack_sat(mu[2], v_c), f16x2_pack_sat(mu_d, v_d));
+    }
+};
+
+// ranked_step's Io on either: the colour mixture, the depth mixture, the
+// augmented one.
+template <int M, class S> struct ColourF16 {
+    S &s;
+    __device__ __forceinline__ void load_means(float (&m)[M][3], int i0) {
+        s.load_c();
+#pragma unroll
+        for (int i = i0; i < M; ++i) {
+            const float2 rg = s.rg(i);
+            m[i][0] = rg.x;
+            m[i][1] = rg.y;
+            m[i][2] = s.mu_b(i);
+        }
+    }
+    __device__ __forceinline__ void put(int r, const float (&mu)[3], float v) { s.put_c(r, mu, v); }
+};
+template <int M, class S> struct DepthF16 {
+    S &s;
+    __device__ __forceinline__ void load_means(float (&m)[M][1], int i0) {
+        s.load_d();
+#pragma unroll
+        for (int i = i0; i < M; ++i)
+            m[i][0] = s.mu_d(i);
+    }
+    __device__ __forceinline__ void put(int r, const float (&mu)[1], float v) {
+        s.put_d(r, mu[0], v);
+    }
+};
+template <int M, class S> struct AugmentedF16 {
+    S &s;
+    __device__ __forceinline__ void load_means(float (&m)[M][4], int i0) {
+        s.load_c();
+#pragma unroll
+        for (int i = i0; i < M; ++i) {
+            const float2 rg = s.rg(i);
+            m[i][0] = rg.x;
+            m[i][1] = rg.y;
+            m[i][2] = s.mu_b(i);
+            m[i][3] = s.mu_d(i);
+        }
+    }
+    __device__ __forceinline__ void put(int r, const float (&mu)[4], float v) {
+        s.put_c(r, mu, v);
+        s.put_d(r, mu[3], 0.f);
+    }
+};
+
+// The two weights of component i as stored (stochastic rounding on request).
+template <int kVariant>
+__device__ __forceinline__ uint32_t pack_weights(const CamView &cv, uint32_t p, int i, float wc,
+                                                 float wd) {
+    const uint32_t sr = kVariant != 0 ? sr_weights(cv, p, i) : 0u;
+    return (kVariant != 0 && sr) ? bf16x2_pack_sr(wc, wd, sr) : bf16x2_pack(wc, wd);
+}
+
+// FP16/BF16 state, the first tick (as first_pixel_f32).
+template <int M, class S, int kVariant>
+__device__ __forceinline__ void first_pixel_f16(const CamView &cv, int64_t p, S &s,
+                                                const float (&xc)[3], uint32_t draw) {
+    const float w0 = 1.0f / (float)M;
+    const bool depth = kVariant != 2 && draw != 0u;
+    const float z = kVariant == 2 ? (draw ? cv.depth_scale * (float)draw : 0.f) : (float)draw;
 #pragma unroll
     for (int i = 0; i < M; ++i)
-        store(i, {c[i].w, c[i].mu[0], c[i].mu[1], c[i].mu[2], c[i].v, d[i].w, d[i].mu[0], d[i].v});
-    cv.fusion[p] = (uint8_t)fb;
-    return (fb & 1u) | ((uint32_t)fgc << 1) | ((uint32_t)fgd << 2);
+        s.store_all(i, pack_weights<kVariant>(cv, (uint32_t)p, i, w0, depth ? w0 : 0.f), xc,
+                    cv.pc.init_var, z, depth ? cv.pd.init_var : 0.f);
+    cv.fusion[p] = kVariant == 2 ? (uint8_t)0u
+                                 : (uint8_t)fuse_list1(0, 0, depth ? kDepthStarted : 0u);
+}
+
+// FP16/BF16 state after the first tick. S: how the state is laid out.
+template <int M, class S, int kVariant>
+__device__ __forceinline__ uint32_t tick_pixel_f16(const CamView &cv, int64_t p, S &s,
+                                                   const float (&xc)[3], uint32_t draw,
+                                                   uint32_t lanes_c) {
+    const uint32_t fb0 = kVariant == 2 ? 0u : cv.fusion[p];
+    s.load();
+    float w[M], v[M], wd[M];
+    if constexpr (kVariant == 2) {
+        s.clear_v_d();
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            w[i] = bf16_lo(s.W[i]);
+            v[i] = s.v_c(i);
+        }
+        const float2 rg = s.rg(0);
+        float mu[4] = {rg.x, rg.y, s.mu_b(0), s.mu_d(0)};
+        const float xa[4] = {xc[0], xc[1], xc[2], draw ? cv.depth_scale * (float)draw : mu[3]};
+        AugmentedF16<M, S> io = {s};
+        const uint32_t f = (uint32_t)ranked_step<M, 4, true>(io, w, v, mu, xa, cv.pc, lanes_c);
+#pragma unroll
+        for (int i = 0; i < M; ++i) // w_d is unused and reads as zero
+            s.store(i, pack_weights<kVariant>(cv, (uint32_t)p, i, w[i], 0.f));
+        cv.fusion[p] = (uint8_t)f;
+        return f | (f << 1) | (f << 2);
+    } else {
+        int fgc, fgd;
+        {
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                w[i] = bf16_lo(s.W[i]);
+                v[i] = s.v_c(i);
+            }
+            const float2 rg = s.rg(0);
+            float mu[3] = {rg.x, rg.y, s.mu_b(0)};
+            ColourF16<M, S> io = {s};
+            fgc = ranked_step<M, 3, (kVariant != 0)>(io, w, v, mu, xc, cv.pc, lanes_c);
+        }
+        // The lanes that run the depth mixture: a reading, and a started model.
+        uint32_t fb = fb0;
+        const uint32_t lanes_d = __ballot_sync(lanes_c, draw != 0u && (fb & kDepthStarted));
+#pragma unroll
+        for (int i = 0; i < M; ++i)
+            wd[i] = bf16_hi(s.W[i]);
+        if (draw == 0u) {
+            fgd = fgc; // no reading: depth model untouched, depth answer = colour
+        } else if (!(fb & kDepthStarted)) {
+            s.load_bd();
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                wd[i] = 1.0f / (float)M;
+                s.put_d(i, (float)draw, cv.pd.init_var);
+            }
+            fb |= kDepthStarted;
+            fgd = 0;
+        } else {
+#pragma unroll
+            for (int i = 0; i < M; ++i)
+                v[i] = s.v_d(i);
+            const float xd[1] = {(float)draw};
+            float mu[1] = {s.mu_d(0)};
+            DepthF16<M, S> io = {s};
+            fgd = ranked_step<M, 1, (kVariant != 0)>(io, wd, v, mu, xd, cv.pd, lanes_d);
+        }
+        fb = fuse_list1(fgc, fgd, fb);
+#pragma unroll
+        for (int i = 0; i < M; ++i)
+            s.store(i, pack_weights<kVariant>(cv, (uint32_t)p, i, w[i], wd[i]));
+        if (fb != fb0)
+            cv.fusion[p] = (uint8_t)fb;
+        return (fb & 1u) | ((uint32_t)fgc << 1) | ((uint32_t)fgd << 2);
+    }
 }
 
 // p: padded linear pixel index (row * w_pad + x). Returns bit 0 fused label,
@@ -840,17 +862,24 @@ __device__ __forceinline__ uint32_t process_pixel(const CamView &cv, int64_t p) 
     const float xc[3] = {(float)cv.rgb[3 * q], (float)cv.rgb[3 * q + 1],
                          (float)cv.rgb[3 * q + 2]};
     const uint32_t draw = cv.depth[q];
-    // First element of the pixel's tile, and the pixel's column in it.
-    const int64_t tb = (int64_t)(p32 / kTile) * (kFields * M * kTile);
+    // The pixel's state tile, and its column in it.
+    const int64_t tile = p32 / kTile;
     const uint32_t t = p32 % kTile;
-    if constexpr (PREC == 0) {
+    if constexpr (PREC == kF32) {
+        const int64_t e0 = tile * (kFields * M * kTile) + t;
         if (cv.first) {
-            first_pixel_f32<M, kVariant>(cv, p, tb + t, xc, draw);
+            first_pixel_f32<M, kVariant>(cv, p, e0, xc, draw);
             return 0u;
         }
-        return tick_pixel_f32<M, kVariant>(cv, p, tb + t, xc, draw, lanes_c);
+        return tick_pixel_f32<M, kVariant>(cv, p, e0, xc, draw, lanes_c);
     } else {
-        return tick_pixel_f16<M, kVariant>(cv, p, tb, t, xc, draw, lanes_c);
+        using S = std::conditional_t<PREC == kF16, PairsF16<M>, GroupsF16<M>>;
+        S s(cv.planes, tile, t);
+        if (cv.first) {
+            first_pixel_f16<M, S, kVariant>(cv, p, s, xc, draw);
+            return 0u;
+        }
+        return tick_pixel_f16<M, S, kVariant>(cv, p, s, xc, draw, lanes_c);
     }
 }
 

@@ -13,8 +13,8 @@ namespace gmmhost {
 cudaError_t launch_tick(const gmmdev::CamView &cv, int threads, cudaStream_t s);
 
 // Block size of the direct tick kernel for gmm_set_kernel's variant: 0 the
-// measured best for the storage precision (FP32: 128; FP16/BF16: 64, two
-// warps of two pixels per thread), 1..4: 256, 128, 64, 32.
+// measured best for the storage precision (FP32: 128; FP16/BF16: 64, 45.7 us
+// against 46.4 with 128 at 1920x1080, M = 5), 1..4: 256, 128, 64, 32.
 inline int direct_threads(int variant, int prec) {
     switch (variant) {
     case 1: return 256;

@@ -2,9 +2,9 @@
 // bit-packed mask, mask packing and confusion counts. (The multi-camera tick
 // is in gmm_pool_kernel.cu.)
 //
-// The tick is a stream over the mixture state: per pixel FP32 state needs
-// about 24 M + 40 bytes of it (what a tick reads and changes, see
-// ranked_update), FP16/BF16 state moves all 32 M; plus 5 bytes of frame, the
+// The tick is a stream over the mixture state: per pixel it needs about
+// 24 M + 40 bytes of FP32 state (what a tick reads and changes, see
+// ranked_step) and half that of FP16/BF16 state, plus 5 bytes of frame, the
 // List-1 byte and 1/8 byte of mask. There is no dense contraction, so there
 // is no tensor-core work; the design goal is full-line coalesced traffic
 // with enough bytes in flight per SM.
@@ -30,8 +30,7 @@ __device__ __forceinline__ void dependent_launch_prologue() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// FP32 state: one thread per padded pixel (n_pad is a multiple of 32: whole
-// warps leave).
+// One thread per padded pixel (n_pad is a multiple of 32: whole warps leave).
 template <int M, int PREC, int V>
 __device__ __forceinline__ void tick_body(const CamView &cv) {
     dependent_launch_prologue();
@@ -42,40 +41,22 @@ __device__ __forceinline__ void tick_body(const CamView &cv) {
     write_mask_words(cv, p >> 5, bits);
 }
 
-// FP16/BF16 state: two pixels per thread, each warp a 64-pixel chunk (lane
-// t takes pixels t and t + 32, so both halves stay coalesced); the second
-// pixel's loads overlap the first one's arithmetic. A half chunk past n_pad
-// is skipped by the whole warp.
-template <int M, int PREC, int V>
-__device__ __forceinline__ void tick_body2(const CamView &cv) {
-    dependent_launch_prologue();
-    const int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 64;
-    if (base >= cv.n_pad)
-        return;
-    const int lane = threadIdx.x & 31;
-    uint32_t bits[2];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        const int64_t p = base + 32 * u + lane;
-        bits[u] = p < cv.n_pad ? process_pixel<M, PREC, V>(cv, p) : 0u;
-    }
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-        if (base + 32 * u < cv.n_pad)
-            write_mask_words(cv, (base >> 5) + u, bits[u]);
-}
-
-// FP32 state: 64 registers and 32 warps per SM at M = 5; 5.9 of the 6.3 TB/s
-// that this mix of reads and partial writes reaches in the pooled kernel, the
-// rest being each launch's ramp and drain (about 7 us). FP16/BF16 state: issue bound; at least 1024 threads per SM. V: process_pixel's variant (the options are separate
-// instantiations, so the default kernels carry none of them). Small CTAs
+// V: process_pixel's variant (the options are separate instantiations, so the
+// default kernels carry none of them). FP32 state: 64 registers and 32 warps
+// per SM at M = 5; 5.9 of the 6.3 TB/s that this mix of reads and partial
+// writes reaches in the pooled kernel, the rest being each launch's ramp and
+// drain (about 7 us). FP16/BF16 state: half the bytes for as many
+// instructions, so issue slots (63% used) and latency share the bound: at
+// least 1024 threads per SM; two pixels per thread spill (1920x1080, M = 5:
+// 53.0 us against 45.7), 80 registers and 24 warps measured 50.3. Small CTAs
 // measured faster than 256 threads: a CTA's slot frees as soon as its own
-// warps finish. A persistent grid-stride form measured slower (its loop
-// costs registers: 66 in FP32, i.e. 3 CTAs of 256 per SM).
+// warps finish. A persistent form fed by bulk copies through shared memory
+// measured slower (73 us against 70 in FP32): a stage waits for the slowest of
+// its warps, and in most tiles one of them goes to memory for a mean.
 template <int M, int V>
-__global__ void __launch_bounds__(256) k_tick_f32(const CamView cv) { tick_body<M, 0, V>(cv); }
-template <int M, int V>
-__global__ void __launch_bounds__(256, 4) k_tick_f16(const CamView cv) { tick_body2<M, 1, V>(cv); }
+__global__ void __launch_bounds__(256) k_tick_f32(const CamView cv) { tick_body<M, kF32, V>(cv); }
+template <int M, int PREC, int V>
+__global__ void __launch_bounds__(256, 4) k_tick_f16(const CamView cv) { tick_body<M, PREC, V>(cv); }
 
 template <int M, int PREC, int V>
 cudaError_t launch_tick_v(const CamView &cv, int threads, cudaStream_t s) {
@@ -83,18 +64,15 @@ cudaError_t launch_tick_v(const CamView &cv, int threads, cudaStream_t s) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)((cv.n_pad + threads - 1) / threads));
     cfg.blockDim = dim3((unsigned)threads);
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (PREC == 0) {
-        cfg.gridDim = dim3((unsigned)((cv.n_pad + threads - 1) / threads));
+    if constexpr (PREC == kF32)
         return cudaLaunchKernelEx(&cfg, k_tick_f32<M, V>, cv);
-    }
-    const int64_t chunks = (cv.n_pad + 63) / 64; // one per warp
-    const int warps = threads / 32;
-    cfg.gridDim = dim3((unsigned)((chunks + warps - 1) / warps));
-    return cudaLaunchKernelEx(&cfg, k_tick_f16<M, V>, cv);
+    else
+        return cudaLaunchKernelEx(&cfg, k_tick_f16<M, PREC, V>, cv);
 }
 
 template <int M, int PREC>
@@ -256,17 +234,23 @@ cudaError_t launch_tick(const CamView &cv, int threads, cudaStream_t s) {
         return cudaSuccess;
     if (threads != 32 && threads != 64 && threads != 128 && threads != 256)
         return cudaErrorInvalidValue;
-    if (cv.prec == 0) {
+    if (cv.prec == kF32) {
         switch (cv.M) {
-        case 3: return launch_tick_t<3, 0>(cv, threads, s);
-        case 4: return launch_tick_t<4, 0>(cv, threads, s);
-        case 5: return launch_tick_t<5, 0>(cv, threads, s);
+        case 3: return launch_tick_t<3, kF32>(cv, threads, s);
+        case 4: return launch_tick_t<4, kF32>(cv, threads, s);
+        case 5: return launch_tick_t<5, kF32>(cv, threads, s);
+        }
+    } else if (cv.prec == kF16) {
+        switch (cv.M) {
+        case 3: return launch_tick_t<3, kF16>(cv, threads, s);
+        case 4: return launch_tick_t<4, kF16>(cv, threads, s);
+        case 5: return launch_tick_t<5, kF16>(cv, threads, s);
         }
     } else {
         switch (cv.M) {
-        case 3: return launch_tick_t<3, 1>(cv, threads, s);
-        case 4: return launch_tick_t<4, 1>(cv, threads, s);
-        case 5: return launch_tick_t<5, 1>(cv, threads, s);
+        case 3: return launch_tick_t<3, kF16Caller>(cv, threads, s);
+        case 4: return launch_tick_t<4, kF16Caller>(cv, threads, s);
+        case 5: return launch_tick_t<5, kF16Caller>(cv, threads, s);
         }
     }
     return cudaErrorInvalidValue;

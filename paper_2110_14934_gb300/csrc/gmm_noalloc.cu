@@ -125,8 +125,10 @@ extern "C" int gmm_apply_open3_noalloc(const gmm_config *cfg, void *state, int f
     if (rc != GMM_OK)
         return rc;
     const Layout L = make_layout(cfg->H, cfg->W, cfg->M, cfg->precision);
-    const gmmdev::CamView v = make_view(*cfg, L, state, rgb8, depth16, scratch, nullptr,
-                                        nullptr, first, 0u);
+    gmmdev::CamView v = make_view(*cfg, L, state, rgb8, depth16, scratch, nullptr, nullptr,
+                                  first, 0u);
+    if (cfg->precision == GMM_PREC_F16)
+        v.prec = gmmdev::kF16Caller; // the layout that gmm.h gives
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaError_t e = gmmhost::launch_tick(v, gmmhost::direct_threads(0, cfg->precision), s);
     if (e == cudaSuccess)

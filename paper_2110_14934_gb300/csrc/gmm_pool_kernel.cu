@@ -73,27 +73,27 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
 constexpr int64_t kPrefetchBudget = 16ll << 20;
 
 // Prefetch the state and List-1 bytes of the first pixels of tile t (camera
-// job) into L2. The state is whole 256-pixel state tiles, one contiguous block
-// of the camera's allocation (which holds every state tile up to n_tiles);
-// the List-1 bytes start at a multiple of 32 and number a multiple of 32.
-template <int PREC>
+// job) into L2: of each 256-pixel state tile the planes that every tick reads,
+// one contiguous block at its head (the camera's allocation holds every state
+// tile up to n_tiles); the List-1 bytes start at a multiple of 32 and number a
+// multiple of 32.
 __device__ __forceinline__ void prefetch_tile(const PoolArgs &a, int64_t t, int job) {
     const CamView &v = a.views[job];
-    const int64_t tile_bytes = (int64_t)kFields * v.M * kTile * (PREC == 0 ? 4 : 2);
-    const int64_t share = kPrefetchBudget / gridDim.x / (tile_bytes + kTile);
+    const int64_t tile_bytes = (int64_t)kFields * v.M * kTile * 2;
+    const uint32_t head = (uint32_t)(2 * v.M + 2) * kTile * 4;
+    const int64_t share = kPrefetchBudget / gridDim.x / (head + kTile);
     const int64_t q0 = (t - a.tile_begin[job]) * a.tile_pixels;
     const int64_t s0 = q0 / kTile;
     const int64_t q1 = min(min(q0 + (int64_t)a.tile_pixels, v.n_pad),
                            (s0 + max(share, (int64_t)1)) * kTile);
     const int64_t s1 = (q1 + kTile - 1) / kTile;
-    prefetch_l2(static_cast<const char *>(v.planes) + s0 * tile_bytes,
-                (uint32_t)((s1 - s0) * tile_bytes));
+    for (int64_t s = s0; s < s1; ++s)
+        prefetch_l2(static_cast<const char *>(v.planes) + s * tile_bytes, head);
     prefetch_l2(v.fusion + q0, (uint32_t)(q1 - q0));
 }
 
 // Take the CTA's next tile from the counter into slot `slot` (thread 0),
 // prefetching its first pixels' state when asked.
-template <int PREC>
 __device__ __forceinline__ void take_next(const PoolArgs &a, int64_t *s_tile, int *s_job,
                                           int slot, bool prefetch) {
     const int64_t tn = atomicAdd(a.counter, 1);
@@ -101,7 +101,7 @@ __device__ __forceinline__ void take_next(const PoolArgs &a, int64_t *s_tile, in
     s_tile[slot] = tn;
     s_job[slot] = jn;
     if (prefetch && tn < a.n_tiles)
-        prefetch_tile<PREC>(a, tn, jn);
+        prefetch_tile(a, tn, jn);
 }
 
 // kAll: tiles may come from cameras that use the options or the
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(256, (PREC == 0 && kAll) ? 3 : 4) k_pool_tick(
     if constexpr (!kPrefetch) {
         for (;;) { // take a tile, publish it, read it, barrier (slot 0 is rewritten)
             if (threadIdx.x == 0)
-                take_next<PREC>(a, s_tile, s_job, 0, false);
+                take_next(a, s_tile, s_job, 0, false);
             __syncthreads();
             const int64_t t = s_tile[0];
             const int job = s_job[0];
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(256, (PREC == 0 && kAll) ? 3 : 4) k_pool_tick(
         }
     }
     if (threadIdx.x == 0)
-        take_next<PREC>(a, s_tile, s_job, 0, false);
+        take_next(a, s_tile, s_job, 0, false);
     __syncthreads();
     for (int k = 0;; k ^= 1) {
         const int64_t t = s_tile[k];
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(256, (PREC == 0 && kAll) ? 3 : 4) k_pool_tick(
         const bool early = a.tile_pixels <= 2 * (int)blockDim.x &&
                            t + 2 * (int64_t)gridDim.x < a.n_tiles;
         if (early && threadIdx.x == 0)
-            take_next<PREC>(a, s_tile, s_job, k ^ 1, true);
+            take_next(a, s_tile, s_job, k ^ 1, true);
         const CamView &cv = a.views[job];
         const int64_t p0 = (t - a.tile_begin[job]) * a.tile_pixels;
         const int64_t p1 = min(p0 + (int64_t)a.tile_pixels, cv.n_pad);
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(256, (PREC == 0 && kAll) ? 3 : 4) k_pool_tick(
         default: pool_tile_v<5, PREC, kAll>(cv, p0, p1); break;
         }
         if (!early && threadIdx.x == 0)
-            take_next<PREC>(a, s_tile, s_job, k ^ 1, false);
+            take_next(a, s_tile, s_job, k ^ 1, false);
         __syncthreads();
     }
 }

@@ -27,8 +27,8 @@ using namespace gmmdev;
 
 namespace {
 
-template <int PREC, int TP> struct Smem;
-template <int TP> struct Smem<0, TP> {
+template <int PREC, int M, int TP> struct Smem;
+template <int M, int TP> struct Smem<0, M, TP> {
     static constexpr int kBytes = 4;
     static __device__ __forceinline__ float ldw(const uint8_t *st, int k, int t) {
         return reinterpret_cast<const float *>(st + k * TP * 4)[t];
@@ -43,13 +43,13 @@ template <int TP> struct Smem<0, TP> {
         reinterpret_cast<float *>(st + k * TP * 4)[t] = v;
     }
 };
-// FP16/BF16: plane k = 8 i + f is slot h16_slot(f) of group h16_group(f) of
-// component i (the layout of gmm_device.cuh; TP pixels per tile).
-template <int TP> struct Smem<1, TP> {
+// FP16/BF16: field f = k & 7 of component k >> 3 is a slot of a plane of pairs
+// (the layout of gmm_device.cuh; TP pixels per tile).
+template <int M, int TP> struct Smem<1, M, TP> {
     static constexpr int kBytes = 2;
     static __device__ __forceinline__ int at(int k, int t) {
         const int f = k & 7;
-        return ((2 * (k >> 3) + h16_group(f)) * TP + t) * 4 + h16_slot(f);
+        return (pair_plane(M, k >> 3, f) * TP + t) * 2 + pair_slot(f);
     }
     static __device__ __forceinline__ float ldw(const uint8_t *st, int k, int t) {
         return __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(st)[at(k, t)]);
@@ -72,7 +72,7 @@ template <int TP> struct Smem<1, TP> {
 template <int M, int D, int PREC, int TP>
 __device__ __forceinline__ int staged_mixture_step(uint8_t *st, int f0, int t,
                                                    const float (&x)[D], const StreamPrm &p) {
-    using A = Smem<PREC, TP>;
+    using A = Smem<PREC, M, TP>;
     float w[M], v[M], mu[M][D];
 #pragma unroll
     for (int i = 0; i < M; ++i) {
@@ -207,7 +207,7 @@ __device__ __forceinline__ int staged_mixture_step(uint8_t *st, int f0, int t,
 template <int M, int PREC>
 __device__ __forceinline__ uint32_t staged_pixel(uint8_t *st, int t, const CamView &cv,
                                                  const float (&xc)[3], uint32_t draw) {
-    using A = Smem<PREC, kTile>;
+    using A = Smem<PREC, M, kTile>;
     uint8_t *fus = st + kFields * M * kTile * A::kBytes;
     uint32_t fb = fus[t];
     const int fgc = staged_mixture_step<M, 3, PREC, kTile>(st, F_WC, t, xc, cv.pc);
@@ -238,7 +238,7 @@ __device__ __forceinline__ uint32_t staged_pixel(uint8_t *st, int t, const CamVi
 // List-1 bytes and, when cv.flags has kStageInputs, its RGB and depth bytes.
 template <int M, int PREC, int ST>
 __global__ void __launch_bounds__(kTile) k_tick_staged(const CamView cv, int *status) {
-    using A = Smem<PREC, kTile>;
+    using A = Smem<PREC, M, kTile>;
     constexpr uint32_t STATE = kFields * M * kTile * A::kBytes; // one tile of planes
     constexpr uint32_t FUS = STATE;                            // List-1 bytes
     constexpr uint32_t RGB = FUS + kTile;                      // 3 bytes per pixel
