@@ -339,11 +339,15 @@ static int pool_tick_impl(gmm_pool *p, bool clear) {
         j = 0;
         tiles = 0;
     };
-    const int groups[3] = {3, 4, 5};
-    for (int gi = 0; gi < (flat ? 3 : 1); ++gi) {
-        group_m = flat ? groups[gi] : 0;
+    // Cameras in order of M: the flat form launches per M; in the persistent
+    // form the CTAs that run together then run one M's body of code (with the
+    // cameras mixed, the bodies of all three evict each other from the
+    // instruction caches), and the longest tiles come first.
+    const int groups[3] = {5, 4, 3};
+    for (int m : groups) {
+        group_m = flat ? m : 0;
         for (PoolCam &c : p->cams) {
-            if (!(c.used && c.submitted) || (group_m && c.cfg.M != group_m))
+            if (!(c.used && c.submitted) || c.cfg.M != m)
                 continue;
             gmmhost::PoolArgs &a = p->h_args[b][li];
             a.views[j] = make_view(c.cfg, c.L, c.arena, c.rgb, c.depth, c.mask, c.fgr, c.fgd,
@@ -354,9 +358,11 @@ static int pool_tick_impl(gmm_pool *p, bool clear) {
             if (++j == gmmhost::kPoolViews)
                 close_launch();
         }
-        if (j > 0)
+        if (flat && j > 0)
             close_launch();
     }
+    if (j > 0)
+        close_launch();
     const int n_launch = li;
     cudaError_t e = cudaSuccess;
     if (clear && tu.active && tu.open.a) { // this tick's start ends the last trial's period
