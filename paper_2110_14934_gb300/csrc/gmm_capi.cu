@@ -4,6 +4,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <cfloat>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -109,6 +110,11 @@ gmmdev::StreamPrm stream_prm(const gmm_config &c, bool depth) {
     p.init_w = c.init_w;
     p.v_min = depth ? c.v_min_d : c.v_min_c;
     p.flags = c.flags & (gmmdev::kRhoEta | gmmdev::kVarPerChannel);
+    // The default FP16/BF16 kernels take variances to be zero or normal: what
+    // float16 stores is, and so is a new one unless its floor or initial value
+    // is not (such a model runs the options' kernels, whose roots take any).
+    if (c.precision == GMM_PREC_F16 && fminf(p.v_min, p.init_var) < FLT_MIN)
+        p.flags |= gmmdev::kTinyVariance;
     return p;
 }
 

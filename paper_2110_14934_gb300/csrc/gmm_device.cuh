@@ -46,6 +46,7 @@ constexpr int kModeAugmented = 2; // CamView.flags: one 4-channel mixture (R, G,
 constexpr int kStochasticWeights = 4; // CamView.flags: BF16 weights stored with stochastic rounding
 constexpr uint32_t kRhoEta = 1u;        // StreamPrm.flags: rho = alpha * eta(x | mu, sigma)
 constexpr uint32_t kVarPerChannel = 2u; // StreamPrm.flags: v is the per-channel variance
+constexpr uint32_t kTinyVariance = 4u;  // StreamPrm.flags: a new variance may be denormal
 
 // Storage of the state, as the kernels' PREC (CamView.prec).
 enum { kF32 = 0, kF16 = 1, kF16Caller = 2 };
@@ -62,7 +63,7 @@ __host__ __device__ constexpr int pair_slot(int f) {
 
 struct StreamPrm {
     float alpha, oma, k2, T, init_var, init_w, v_min;
-    uint32_t flags; // kRhoEta | kVarPerChannel
+    uint32_t flags; // kRhoEta | kVarPerChannel | kTinyVariance
 };
 
 // Learning rate of the matched component: alpha, or with kRhoEta
@@ -186,8 +187,21 @@ __device__ __forceinline__ uint32_t f16x2_set_hi(uint32_t pair, float hi) {
 // included), puts the lower stored rank first: a total order, under which the
 // network's result is the stable sort. (Two values that close lie well inside
 // the 1e-5 margin at which a decision counts as near its threshold.)
+// kNormalV: v is zero or a normal number, so the root needs no care for
+// denormal ones (three instructions each; the result is the same).
+template <bool kNormalV> __device__ __forceinline__ uint32_t rank_bits(float w, float v) {
+    float r;
+    if (kNormalV)
+        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    else
+        r = rsqrtf(v);
+    return __float_as_uint(w * r);
+}
+__device__ __forceinline__ uint32_t rank_key(uint32_t bits, int i) {
+    return (bits & ~7u) | (7u - (uint32_t)i);
+}
 __device__ __forceinline__ uint32_t rank_key(float w, float v, int i) {
-    return (__float_as_uint(w * rsqrtf(v)) & ~7u) | (7u - (uint32_t)i);
+    return rank_key(rank_bits<false>(w, v), i);
 }
 
 template <int D> struct Comp {
@@ -296,7 +310,7 @@ __device__ __forceinline__ float moved_component(float (&mu)[D], float v, const 
     return fmaxf(p.v_min, fmaf(orho, v, rho * (kOptions ? var_sample<D>(p, d2n) : d2n)));
 }
 
-template <int M, int D, bool kOptions, class Io>
+template <int M, int D, bool kOptions, bool kNormalV, class Io>
 __device__ __forceinline__ int ranked_step(Io &io, float (&w)[M], float (&v)[M], float (&mu)[D],
                                            const float (&x)[D], const StreamPrm &p,
                                            uint32_t lanes) {
@@ -371,14 +385,14 @@ __device__ __forceinline__ int ranked_step(Io &io, float (&w)[M], float (&v)[M],
     // lane's components are already in non-increasing key order (the usual
     // case), the stable network would leave them as they are, so the warp
     // skips it and the changed component keeps its rank.
-    uint32_t key[M];
+    uint32_t bits[M];
     bool sorted = true;
 #pragma unroll
     for (int i = 0; i < M; ++i) {
         w[i] *= inv;
-        key[i] = rank_key(w[i], v[i], i);
-        if (i > 0)
-            sorted = sorted && !(key[i] > key[i - 1]);
+        bits[i] = rank_bits<kNormalV>(w[i], v[i]);
+        if (i > 0) // rank_key(bits[i], i) > rank_key(bits[i - 1], i - 1)
+            sorted = sorted && !(bits[i] > (bits[i - 1] | 7u));
     }
     int rank = jj; // the changed component's rank after the update
     if (__any_sync(lanes, !sorted)) {
@@ -388,7 +402,7 @@ __device__ __forceinline__ int ranked_step(Io &io, float (&w)[M], float (&v)[M],
         Comp<D> c[M];
 #pragma unroll
         for (int i = 0; i < M; ++i) {
-            c[i].key = key[i];
+            c[i].key = rank_key(bits[i], i);
             c[i].w = w[i];
             c[i].v = v[i];
 #pragma unroll
@@ -405,8 +419,9 @@ __device__ __forceinline__ int ranked_step(Io &io, float (&w)[M], float (&v)[M],
             if (id == jj || id != r)
                 io.put(r, c[r].mu, c[r].v);
         }
-    } else if (all_best) {
+    } else if (all_best) { // background: no weight comes before rank 0
         io.put(0, mu, v[0]);
+        return 0;
     } else {
 #pragma unroll
         for (int r = 0; r < M; ++r)
@@ -517,7 +532,7 @@ __device__ __forceinline__ uint32_t tick_pixel_f32(const CamView &cv, int64_t p,
         float mu[4] = {at(0, F_MUR), at(0, F_MUG), at(0, F_MUB), at(0, F_MUD)};
         const float xa[4] = {xc[0], xc[1], xc[2], draw ? cv.depth_scale * (float)draw : mu[3]};
         PlanesF32<M, 4, F_MUR, F_VC> io = {b};
-        const uint32_t f = (uint32_t)ranked_step<M, 4, true>(io, w, v, mu, xa, cv.pc, lanes_c);
+        const uint32_t f = (uint32_t)ranked_step<M, 4, true, false>(io, w, v, mu, xa, cv.pc, lanes_c);
 #pragma unroll
         for (int r = 0; r < M; ++r)
             at(r, F_WC) = w[r];
@@ -533,7 +548,7 @@ __device__ __forceinline__ uint32_t tick_pixel_f32(const CamView &cv, int64_t p,
             vd[i] = at(i, F_VD);
         }
         PlanesF32<M, 3, F_MUR, F_VC> colour = {b};
-        const int fgc = ranked_step<M, 3, (kVariant != 0)>(colour, w, v, mu, xc, cv.pc, lanes_c);
+        const int fgc = ranked_step<M, 3, (kVariant != 0), false>(colour, w, v, mu, xc, cv.pc, lanes_c);
 #pragma unroll
         for (int r = 0; r < M; ++r)
             at(r, F_WC) = w[r];
@@ -555,7 +570,7 @@ __device__ __forceinline__ uint32_t tick_pixel_f32(const CamView &cv, int64_t p,
         } else {
             const float xd[1] = {(float)draw};
             PlanesF32<M, 1, F_MUD, F_VD> depth = {b};
-            fgd = ranked_step<M, 1, (kVariant != 0)>(depth, wd, vd, mud, xd, cv.pd, lanes_d);
+            fgd = ranked_step<M, 1, (kVariant != 0), false>(depth, wd, vd, mud, xd, cv.pd, lanes_d);
 #pragma unroll
             for (int r = 0; r < M; ++r)
                 at(r, F_WD) = wd[r];
@@ -625,11 +640,22 @@ template <int M> struct PairsF16 {
             }
         }
     }
-    __device__ __forceinline__ void store(int i, uint32_t w) const {
-        at(2 * i) = w;
-        if (changed >> i & 1u) {
-            at(2 * i + 1) = V[i];
-            at(2 * M + 2 * i + 1) = BD[i];
+    __device__ __forceinline__ void store(const uint32_t (&w)[M]) const {
+#pragma unroll
+        for (int i = 0; i < M; ++i)
+            at(2 * i) = w[i];
+        if (changed & 1u) {
+            at(1) = V[0];
+            at(2 * M + 1) = BD[0];
+        }
+        if (changed > 1u) {
+#pragma unroll
+            for (int i = 1; i < M; ++i) {
+                if (changed >> i & 1u) {
+                    at(2 * i + 1) = V[i];
+                    at(2 * M + 2 * i + 1) = BD[i];
+                }
+            }
         }
     }
     // The first tick: component i whole.
@@ -687,10 +713,18 @@ template <int M> struct GroupsF16 {
             }
         }
     }
-    __device__ __forceinline__ void store(int i, uint32_t w) const {
-        b[2 * i * kTile] = make_uint2(w, RG[i]);
-        if (changed >> i & 1u)
-            b[(2 * i + 1) * kTile] = make_uint2(BV[i], DV[i]);
+    __device__ __forceinline__ void store(const uint32_t (&w)[M]) const {
+#pragma unroll
+        for (int i = 0; i < M; ++i)
+            b[2 * i * kTile] = make_uint2(w[i], RG[i]);
+        if (changed & 1u)
+            b[kTile] = make_uint2(BV[0], DV[0]);
+        if (changed > 1u) {
+#pragma unroll
+            for (int i = 1; i < M; ++i)
+                if (changed >> i & 1u)
+                    b[(2 * i + 1) * kTile] = make_uint2(BV[i], DV[i]);
+        }
     }
     __device__ __forceinline__ void store_all(int i, uint32_t w, const float *mu, float v_c,
                                               float mu_d, float v_d) const {
@@ -788,10 +822,12 @@ __device__ __forceinline__ uint32_t tick_pixel_f16(const CamView &cv, int64_t p,
         float mu[4] = {rg.x, rg.y, s.mu_b(0), s.mu_d(0)};
         const float xa[4] = {xc[0], xc[1], xc[2], draw ? cv.depth_scale * (float)draw : mu[3]};
         AugmentedF16<M, S> io = {s};
-        const uint32_t f = (uint32_t)ranked_step<M, 4, true>(io, w, v, mu, xa, cv.pc, lanes_c);
+        const uint32_t f = (uint32_t)ranked_step<M, 4, true, false>(io, w, v, mu, xa, cv.pc, lanes_c);
+        uint32_t packed[M]; // w_d is unused and reads as zero
 #pragma unroll
-        for (int i = 0; i < M; ++i) // w_d is unused and reads as zero
-            s.store(i, pack_weights<kVariant>(cv, (uint32_t)p, i, w[i], 0.f));
+        for (int i = 0; i < M; ++i)
+            packed[i] = pack_weights<kVariant>(cv, (uint32_t)p, i, w[i], 0.f);
+        s.store(packed);
         cv.fusion[p] = (uint8_t)f;
         return f | (f << 1) | (f << 2);
     } else {
@@ -805,7 +841,7 @@ __device__ __forceinline__ uint32_t tick_pixel_f16(const CamView &cv, int64_t p,
             const float2 rg = s.rg(0);
             float mu[3] = {rg.x, rg.y, s.mu_b(0)};
             ColourF16<M, S> io = {s};
-            fgc = ranked_step<M, 3, (kVariant != 0)>(io, w, v, mu, xc, cv.pc, lanes_c);
+            fgc = ranked_step<M, 3, (kVariant != 0), (kVariant == 0)>(io, w, v, mu, xc, cv.pc, lanes_c);
         }
         // The lanes that run the depth mixture: a reading, and a started model.
         uint32_t fb = fb0;
@@ -831,12 +867,14 @@ __device__ __forceinline__ uint32_t tick_pixel_f16(const CamView &cv, int64_t p,
             const float xd[1] = {(float)draw};
             float mu[1] = {s.mu_d(0)};
             DepthF16<M, S> io = {s};
-            fgd = ranked_step<M, 1, (kVariant != 0)>(io, wd, v, mu, xd, cv.pd, lanes_d);
+            fgd = ranked_step<M, 1, (kVariant != 0), (kVariant == 0)>(io, wd, v, mu, xd, cv.pd, lanes_d);
         }
         fb = fuse_list1(fgc, fgd, fb);
+        uint32_t packed[M];
 #pragma unroll
         for (int i = 0; i < M; ++i)
-            s.store(i, pack_weights<kVariant>(cv, (uint32_t)p, i, w[i], wd[i]));
+            packed[i] = pack_weights<kVariant>(cv, (uint32_t)p, i, w[i], wd[i]);
+        s.store(packed);
         if (fb != fb0)
             cv.fusion[p] = (uint8_t)fb;
         return (fb & 1u) | ((uint32_t)fgc << 1) | ((uint32_t)fgd << 2);
@@ -880,25 +918,6 @@ __device__ __forceinline__ uint32_t process_pixel(const CamView &cv, int64_t p) 
             return 0u;
         }
         return tick_pixel_f16<M, S, kVariant>(cv, p, s, xc, draw, lanes_c);
-    }
-}
-
-// All 32 lanes of the warp call this for 32 consecutive padded pixels
-// starting at a multiple of 32 (word index wi).
-__device__ __forceinline__ void write_mask_words(const CamView &cv, int64_t wi, uint32_t bits) {
-    const uint32_t F = __ballot_sync(0xffffffffu, bits & 1u);
-    const bool lane0 = (threadIdx.x & 31u) == 0u;
-    if (lane0)
-        cv.mask[wi] = F;
-    if (cv.fg_rgb) { // uniform: the whole warp takes it or not
-        const uint32_t fc = __ballot_sync(0xffffffffu, bits & 2u);
-        if (lane0)
-            cv.fg_rgb[wi] = fc;
-    }
-    if (cv.fg_d) {
-        const uint32_t fd = __ballot_sync(0xffffffffu, bits & 4u);
-        if (lane0)
-            cv.fg_d[wi] = fd;
     }
 }
 

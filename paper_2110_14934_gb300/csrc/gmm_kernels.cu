@@ -42,21 +42,19 @@ __device__ __forceinline__ void tick_body(const CamView &cv) {
 }
 
 // V: process_pixel's variant (the options are separate instantiations, so the
-// default kernels carry none of them). FP32 state: 64 registers and 32 warps
-// per SM at M = 5; 5.9 of the 6.3 TB/s that this mix of reads and partial
-// writes reaches in the pooled kernel, the rest being each launch's ramp and
-// drain (about 7 us). FP16/BF16 state: half the bytes for as many
-// instructions, so issue slots (63% used) and latency share the bound: at
-// least 1024 threads per SM; two pixels per thread spill (1920x1080, M = 5:
-// 53.0 us against 45.7), 80 registers and 24 warps measured 50.3. Small CTAs
+// default kernels carry none of them). The kernels wait for memory more than
+// for anything else, so warps count: 40 per SM (48 registers, small spills)
+// measured 63.8 us against 64.5 with 32 at 1920x1080, M = 5, FP32, and 43.2
+// against 44.4 in FP16/BF16 (48 warps: 47.0; two pixels per thread, which
+// spill: 53.0). Small CTAs
 // measured faster than 256 threads: a CTA's slot frees as soon as its own
 // warps finish. A persistent form fed by bulk copies through shared memory
 // measured slower (73 us against 70 in FP32): a stage waits for the slowest of
 // its warps, and in most tiles one of them goes to memory for a mean.
 template <int M, int V>
-__global__ void __launch_bounds__(256) k_tick_f32(const CamView cv) { tick_body<M, kF32, V>(cv); }
+__global__ void __launch_bounds__(256, 5) k_tick_f32(const CamView cv) { tick_body<M, kF32, V>(cv); }
 template <int M, int PREC, int V>
-__global__ void __launch_bounds__(256, 4) k_tick_f16(const CamView cv) { tick_body<M, PREC, V>(cv); }
+__global__ void __launch_bounds__(256, 5) k_tick_f16(const CamView cv) { tick_body<M, PREC, V>(cv); }
 
 template <int M, int PREC, int V>
 cudaError_t launch_tick_v(const CamView &cv, int threads, cudaStream_t s) {

@@ -106,9 +106,9 @@ __device__ __forceinline__ void take_next(const PoolArgs &a, int64_t *s_tile, in
 
 // kAll: tiles may come from cameras that use the options or the
 // augmentation alternative (launched only when such a camera is in the tick).
-// Registers: 64 in both precisions (32 resident warps per SM; FP32 at 72,
-// 28 warps, measured 0.8% slower on the 64-camera mix), except the FP32
-// instance that also handles the options, which keeps room to avoid spills.
+// Registers: FP32 64 (32 resident warps per SM), the instance that also
+// handles the options 80; FP16/BF16 48 (40 warps; it spills a little, and 24
+// cameras of odd sizes measure 340 us against 343 with 64 registers).
 // FP32 state, the instance that also handles the options, and FP16/BF16
 // pools that turned the prefetch off (kPF = false): thread 0 takes a tile
 // from the counter and publishes it between two barriers. Otherwise, in
@@ -125,7 +125,7 @@ __device__ __forceinline__ void take_next(const PoolArgs &a, int64_t *s_tile, in
 // is written only after the barrier that ended the tile at whose start every
 // thread last read it.
 template <int PREC, bool kAll, bool kPF = true>
-__global__ void __launch_bounds__(256, (PREC == 0 && kAll) ? 3 : 4) k_pool_tick() {
+__global__ void __launch_bounds__(256, PREC != 0 ? 5 : kAll ? 3 : 4) k_pool_tick() {
     constexpr bool kPrefetch = PREC != 0 && !kAll && kPF;
     const PoolArgs &a = c_pool;
     __shared__ int64_t s_tile[2];
