@@ -921,4 +921,46 @@ __device__ __forceinline__ uint32_t process_pixel(const CamView &cv, int64_t p) 
     }
 }
 
+// Move what a tick always reads of a warp's 32 pixels (p: this lane's padded
+// pixel, consecutive from a multiple of 32) closer, one 128-byte line per
+// lane: a hint, which reads nothing itself.
+template <int M, int PREC>
+__device__ __forceinline__ void prefetch_pixels(const CamView &cv, int64_t p) {
+    const uint32_t p32 = (uint32_t)p, lane = p32 & 31u, t = p32 % kTile - lane;
+    const char *tile = static_cast<const char *>(cv.planes) +
+                       (int64_t)(p32 / kTile) * (kFields * M * kTile * (PREC == kF32 ? 4 : 2));
+    uint32_t off;
+    constexpr uint32_t kLines = PREC == kF32 ? 4 * M + 4 : PREC == kF16 ? 2 * M + 2 : 4 * M;
+    if (PREC == kF32) { // w_c, v_c, w_d, v_d of every component, the means of component 0
+        const uint32_t i = lane < 4 * M ? lane >> 2 : 0u;
+        const uint32_t f = (lane < 4 * M ? 0x7540u : 0x6321u) >> (4 * (lane & 3u)) & 15u;
+        off = ((kFields * i + f) * kTile + t) * 4;
+    } else if (PREC == kF16) { // the planes at the head of the tile
+        off = (lane * kTile + t) * 4;
+    } else { // every group, two lines each
+        off = ((lane >> 1) * kTile + t) * 8 + (lane & 1u) * 128;
+    }
+    if (lane < kLines)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(tile + off));
+}
+
+// All 32 lanes of the warp call this for 32 consecutive padded pixels
+// starting at a multiple of 32 (word index wi).
+__device__ __forceinline__ void write_mask_words(const CamView &cv, int64_t wi, uint32_t bits) {
+    const uint32_t F = __ballot_sync(0xffffffffu, bits & 1u);
+    const bool lane0 = (threadIdx.x & 31u) == 0u;
+    if (lane0)
+        cv.mask[wi] = F;
+    if (cv.fg_rgb) { // uniform: the whole warp takes it or not
+        const uint32_t fc = __ballot_sync(0xffffffffu, bits & 2u);
+        if (lane0)
+            cv.fg_rgb[wi] = fc;
+    }
+    if (cv.fg_d) {
+        const uint32_t fd = __ballot_sync(0xffffffffu, bits & 4u);
+        if (lane0)
+            cv.fg_d[wi] = fd;
+    }
+}
+
 } // namespace gmmdev

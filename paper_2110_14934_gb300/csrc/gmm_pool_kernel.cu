@@ -25,7 +25,12 @@ __constant__ PoolArgs c_pool;
 template <int M, int PREC, int V>
 __device__ __forceinline__ void pool_tile(const CamView &cv, int64_t p0, int64_t p1) {
     for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-        // p1 - p0 is a multiple of 32 and blockDim too: warps stay whole.
+        // p1 - p0 is a multiple of 32 and blockDim too: warps stay whole. The
+        // state of the CTA's next pixels moves towards L2 meanwhile (64 FP32
+        // cameras 1361 -> 1279 us, 24 FP16/BF16 ones of odd sizes 340 -> 330;
+        // two steps ahead 1338 and 337, with the List-1 bytes 1309 and 333).
+        if (p + blockDim.x < p1)
+            prefetch_pixels<M, PREC>(cv, p + blockDim.x);
         const uint32_t bits = process_pixel<M, PREC, V>(cv, p);
         write_mask_words(cv, p >> 5, bits);
     }
