@@ -30,31 +30,64 @@ __device__ __forceinline__ void dependent_launch_prologue() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// One thread per padded pixel (n_pad is a multiple of 32: whole warps leave).
-template <int M, int PREC, int V>
-__device__ __forceinline__ void tick_body(const CamView &cv) {
+// A CTA ticks one run of blockDim padded pixels, one pixel per thread (n_pad
+// is a multiple of 32: whole warps leave), or, kLoop, `runs` consecutive ones,
+// moving the next run's state towards L2 while it ticks one.
+template <int M, int PREC, int V, bool kLoop>
+__device__ __forceinline__ void tick_body(const CamView &cv, int runs) {
     dependent_launch_prologue();
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= cv.n_pad)
+    int64_t p = (int64_t)blockIdx.x * blockDim.x * (kLoop ? runs : 1) + threadIdx.x;
+    if (!kLoop) {
+        if (p >= cv.n_pad)
+            return;
+        const uint32_t bits = process_pixel<M, PREC, V>(cv, p);
+        write_mask_words(cv, p >> 5, bits);
         return;
-    const uint32_t bits = process_pixel<M, PREC, V>(cv, p);
-    write_mask_words(cv, p >> 5, bits);
+    }
+    for (int k = 0; k < runs && p < cv.n_pad; ++k, p += blockDim.x) {
+        if (k + 1 < runs && p + blockDim.x < cv.n_pad)
+            prefetch_pixels<M, PREC>(cv, p + blockDim.x);
+        const uint32_t bits = process_pixel<M, PREC, V>(cv, p);
+        write_mask_words(cv, p >> 5, bits);
+    }
 }
 
 // V: process_pixel's variant (the options are separate instantiations, so the
 // default kernels carry none of them). The kernels wait for memory more than
-// for anything else, so warps count: 40 per SM (48 registers, small spills)
-// measured 63.8 us against 64.5 with 32 at 1920x1080, M = 5, FP32, and 43.2
-// against 44.4 in FP16/BF16 (48 warps: 47.0; two pixels per thread, which
-// spill: 53.0). Small CTAs
-// measured faster than 256 threads: a CTA's slot frees as soon as its own
-// warps finish. A persistent form fed by bulk copies through shared memory
-// measured slower (73 us against 70 in FP32): a stage waits for the slowest of
-// its warps, and in most tiles one of them goes to memory for a mean.
-template <int M, int V>
-__global__ void __launch_bounds__(256, 5) k_tick_f32(const CamView cv) { tick_body<M, kF32, V>(cv); }
-template <int M, int PREC, int V>
-__global__ void __launch_bounds__(256, 5) k_tick_f16(const CamView cv) { tick_body<M, PREC, V>(cv); }
+// for anything else (issue slots about 60% used in FP16/BF16, less in FP32),
+// so warps count: 40 per SM (48 registers, small spills) measured 63.8 us
+// against 64.5 with 32 at 1920x1080, M = 5, FP32, and 43.2 against 44.4 in
+// FP16/BF16 (48 warps: 47.0). Two pixels per thread spill (FP16/BF16 53.0);
+// a persistent form fed by bulk copies through shared memory measured slower
+// (73 against 70 at the time: a stage waits for the slowest of its warps, and
+// in most tiles one of them goes to memory for a mean). Small CTAs measured
+// faster than 256 threads: a CTA's slot frees as soon as its own warps finish.
+// The looping form holds more values across a pixel: 64 registers in FP32 and
+// for M = 5.
+template <int M, int PREC, bool kLoop> struct TickBounds {
+    static constexpr int kCtas = kLoop && (PREC == kF32 || M == 5) ? 4 : 5; // of 256 threads
+};
+template <int M, int PREC, int V, bool kLoop>
+__global__ void __launch_bounds__(256, (TickBounds<M, PREC, kLoop>::kCtas))
+    k_tick(const CamView cv, int runs) {
+    tick_body<M, PREC, V, kLoop>(cv, runs);
+}
+
+// Runs per CTA. Looping saves CTA turnover and hides the next run's state
+// behind the current one, but leaves fewer CTAs to even out the end of the
+// launch: it pays from about a dozen waves of a GB300's 152 SMs x 1024
+// threads on. Measured (us; 1, 2, 4 runs): FP32 1280x720 M = 3 options 26.3,
+// 27.9, 30.1; 1920x1080 M = 5 63.6, 62.7, 64.3; 2560x1440 M = 4 95.8, 92.2,
+// 93.2; 3840x2160 M = 5 238, 227, 227; FP16/BF16 1920x1080 M = 3 35.5, 33.7,
+// 33.8; 2560x1440 M = 4 66.7, 64.6, 63.7; 3840x2160 M = 3 133.8, 117.6, 115.7;
+// M = 5 (whose looping form has 32 warps per SM against 40) 1920x1080 43.2,
+// 44.4, 44.7; 3840x2160 162.8, 154.6, 150.7.
+template <int M, int PREC> int tick_runs(int64_t n_pad) {
+    const int64_t waves = n_pad / (152 * 1024);
+    if (waves >= 32)
+        return 4;
+    return waves >= (PREC != kF32 && M == 5 ? 20 : 12) ? 2 : 1;
+}
 
 template <int M, int PREC, int V>
 cudaError_t launch_tick_v(const CamView &cv, int threads, cudaStream_t s) {
@@ -62,15 +95,15 @@ cudaError_t launch_tick_v(const CamView &cv, int threads, cudaStream_t s) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)((cv.n_pad + threads - 1) / threads));
+    const int runs = tick_runs<M, PREC>(cv.n_pad);
+    const int64_t px = (int64_t)threads * runs;
+    cfg.gridDim = dim3((unsigned)((cv.n_pad + px - 1) / px));
     cfg.blockDim = dim3((unsigned)threads);
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if constexpr (PREC == kF32)
-        return cudaLaunchKernelEx(&cfg, k_tick_f32<M, V>, cv);
-    else
-        return cudaLaunchKernelEx(&cfg, k_tick_f16<M, PREC, V>, cv);
+    return runs > 1 ? cudaLaunchKernelEx(&cfg, k_tick<M, PREC, V, true>, cv, runs)
+                    : cudaLaunchKernelEx(&cfg, k_tick<M, PREC, V, false>, cv, runs);
 }
 
 template <int M, int PREC>
