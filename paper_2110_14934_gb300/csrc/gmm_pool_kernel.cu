@@ -111,9 +111,9 @@ __device__ __forceinline__ void take_next(const PoolArgs &a, int64_t *s_tile, in
 
 // kAll: tiles may come from cameras that use the options or the
 // augmentation alternative (launched only when such a camera is in the tick).
-// Registers: FP32 64 (32 resident warps per SM), the instance that also
-// handles the options 80; FP16/BF16 48 (40 warps; it spills a little, and 24
-// cameras of odd sizes measure 340 us against 343 with 64 registers).
+// Registers: 64 (32 resident warps per SM; FP16/BF16 at 48 and 40 warps spills
+// and measures 331 us against 322 on 24 cameras of odd sizes), the FP32
+// instance that also handles the options 80.
 // FP32 state, the instance that also handles the options, and FP16/BF16
 // pools that turned the prefetch off (kPF = false): thread 0 takes a tile
 // from the counter and publishes it between two barriers. Otherwise, in
@@ -130,7 +130,7 @@ __device__ __forceinline__ void take_next(const PoolArgs &a, int64_t *s_tile, in
 // is written only after the barrier that ended the tile at whose start every
 // thread last read it.
 template <int PREC, bool kAll, bool kPF = true>
-__global__ void __launch_bounds__(256, PREC != 0 ? 5 : kAll ? 3 : 4) k_pool_tick() {
+__global__ void __launch_bounds__(256, PREC == 0 && kAll ? 3 : 4) k_pool_tick() {
     constexpr bool kPrefetch = PREC != 0 && !kAll && kPF;
     const PoolArgs &a = c_pool;
     __shared__ int64_t s_tile[2];
