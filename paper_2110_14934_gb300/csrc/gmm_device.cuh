@@ -924,7 +924,7 @@ __device__ __forceinline__ uint32_t process_pixel(const CamView &cv, int64_t p) 
 // Move what a tick always reads of a warp's 32 pixels (p: this lane's padded
 // pixel, consecutive from a multiple of 32) closer, one 128-byte line per
 // lane: a hint, which reads nothing itself.
-template <int M, int PREC>
+template <int M, int PREC, int V>
 __device__ __forceinline__ void prefetch_pixels(const CamView &cv, int64_t p) {
     const uint32_t p32 = (uint32_t)p, lane = p32 & 31u, t = p32 % kTile - lane;
     const char *tile = static_cast<const char *>(cv.planes) +
@@ -940,7 +940,8 @@ __device__ __forceinline__ void prefetch_pixels(const CamView &cv, int64_t p) {
     } else { // every group, two lines each
         off = ((lane >> 1) * kTile + t) * 8 + (lane & 1u) * 128;
     }
-    if (lane < kLines)
+    const bool unused = PREC == kF32 && V == 2 && lane < 4 * M && (lane & 2u); // w_d, v_d
+    if (lane < kLines && !unused)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(tile + off));
 }
 

@@ -32,11 +32,15 @@ __device__ __forceinline__ void dependent_launch_prologue() {
 
 // A CTA ticks one run of blockDim padded pixels, one pixel per thread (n_pad
 // is a multiple of 32: whole warps leave), or, kLoop, `runs` consecutive ones,
-// moving the next run's state towards L2 while it ticks one.
+// moving the next run's state towards L2 while it ticks one. The first `early`
+// CTAs, which the hardware may schedule while the kernel before this one
+// drains, move their first run's state before they wait for that kernel.
 template <int M, int PREC, int V, bool kLoop>
-__device__ __forceinline__ void tick_body(const CamView &cv, int runs) {
-    dependent_launch_prologue();
+__device__ __forceinline__ void tick_body(const CamView &cv, int runs, int early) {
     int64_t p = (int64_t)blockIdx.x * blockDim.x * (kLoop ? runs : 1) + threadIdx.x;
+    if (PREC != kF16 && (int)blockIdx.x < early && p < cv.n_pad)
+        prefetch_pixels<M, PREC, V>(cv, p);
+    dependent_launch_prologue();
     if (!kLoop) {
         if (p >= cv.n_pad)
             return;
@@ -46,7 +50,7 @@ __device__ __forceinline__ void tick_body(const CamView &cv, int runs) {
     }
     for (int k = 0; k < runs && p < cv.n_pad; ++k, p += blockDim.x) {
         if (k + 1 < runs && p + blockDim.x < cv.n_pad)
-            prefetch_pixels<M, PREC>(cv, p + blockDim.x);
+            prefetch_pixels<M, PREC, V>(cv, p + blockDim.x);
         const uint32_t bits = process_pixel<M, PREC, V>(cv, p);
         write_mask_words(cv, p >> 5, bits);
     }
@@ -69,8 +73,8 @@ template <int M, int PREC, bool kLoop> struct TickBounds {
 };
 template <int M, int PREC, int V, bool kLoop>
 __global__ void __launch_bounds__(256, (TickBounds<M, PREC, kLoop>::kCtas))
-    k_tick(const CamView cv, int runs) {
-    tick_body<M, PREC, V, kLoop>(cv, runs);
+    k_tick(const CamView cv, int runs, int early) {
+    tick_body<M, PREC, V, kLoop>(cv, runs, early);
 }
 
 // Runs per CTA. Looping saves CTA turnover and hides the next run's state
@@ -97,13 +101,21 @@ cudaError_t launch_tick_v(const CamView &cv, int threads, cudaStream_t s) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     const int runs = tick_runs<M, PREC>(cv.n_pad);
     const int64_t px = (int64_t)threads * runs;
+    // Two waves of CTAs. An opening's few CTAs leave HBM idle, and so does the
+    // end of a tick: with an opening after each tick FP32 1021x767 M = 4 26.7 ->
+    // 25.2 us, 1280x720 M = 3 options 26.0 -> 25.1, caller-owned FP16/BF16
+    // 1280x720 M = 4 22.1 -> 21.3; ticks alone FP32 1920x1080 M = 5 62.6 ->
+    // 62.0. The FP16/BF16 handles' kernel loses by it (1920x1080 M = 5 43.1 ->
+    // 46.5 us: more spills, and the state it would move is a smaller part of
+    // its time), and does without.
+    const int early = 152 * 2560 / threads;
     cfg.gridDim = dim3((unsigned)((cv.n_pad + px - 1) / px));
     cfg.blockDim = dim3((unsigned)threads);
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return runs > 1 ? cudaLaunchKernelEx(&cfg, k_tick<M, PREC, V, true>, cv, runs)
-                    : cudaLaunchKernelEx(&cfg, k_tick<M, PREC, V, false>, cv, runs);
+    return runs > 1 ? cudaLaunchKernelEx(&cfg, k_tick<M, PREC, V, true>, cv, runs, early)
+                    : cudaLaunchKernelEx(&cfg, k_tick<M, PREC, V, false>, cv, runs, early);
 }
 
 template <int M, int PREC>

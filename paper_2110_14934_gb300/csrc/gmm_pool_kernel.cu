@@ -30,7 +30,7 @@ __device__ __forceinline__ void pool_tile(const CamView &cv, int64_t p0, int64_t
         // cameras 1361 -> 1279 us, 24 FP16/BF16 ones of odd sizes 340 -> 330;
         // two steps ahead 1338 and 337, with the List-1 bytes 1309 and 333).
         if (p + blockDim.x < p1)
-            prefetch_pixels<M, PREC>(cv, p + blockDim.x);
+            prefetch_pixels<M, PREC, V>(cv, p + blockDim.x);
         const uint32_t bits = process_pixel<M, PREC, V>(cv, p);
         write_mask_words(cv, p >> 5, bits);
     }
