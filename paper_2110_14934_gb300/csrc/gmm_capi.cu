@@ -394,6 +394,7 @@ struct gmm_ctx {
     long long slot_ticket[GMM_PIPE_DEPTH] = {-1, -1, -1};
     long long next_ticket = 0;
     long long done_upto = -1;
+    cudaEvent_t ev_host = nullptr; // end of a tick on host buffers in place
     // tick kernel selection and the staged kernel's wait-status word
     int kernel = GMM_KERNEL_DIRECT, variant = 0, ctas_per_sm = 0;
     int *d_status = nullptr;
@@ -635,8 +636,64 @@ int gmm_pipe_wait(gmm_t *h, long long ticket, int timeout_ms) {
     return rc;
 }
 
+// Whether the tick may read the frame from, and write the mask to, these host
+// buffers in place: page-locked memory mapped at the same address, aligned as
+// the kernels need it, the mask apart from the frame.
+static bool in_place(const gmm_ctx *h, const uint8_t *rgb, const uint16_t *depth,
+                     const uint32_t *mask) {
+    const size_t N = (size_t)h->cfg.H * h->cfg.W;
+    const uintptr_t r = reinterpret_cast<uintptr_t>(rgb), d = reinterpret_cast<uintptr_t>(depth),
+                    m = reinterpret_cast<uintptr_t>(mask),
+                    m1 = m + (size_t)h->cfg.H * h->L.wpr * 4;
+    if (d % 2 || m % 4 || (r < m1 && m < r + 3 * N) || (d < m1 && m < d + 2 * N))
+        return false;
+    for (const void *p : {static_cast<const void *>(rgb), static_cast<const void *>(depth),
+                          static_cast<const void *>(mask)}) {
+        cudaPointerAttributes a;
+        if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (a.type != cudaMemoryTypeHost || a.devicePointer != p)
+            return false;
+    }
+    return true;
+}
+
+// With page-locked buffers and no queued frame in flight, the tick works on
+// the host's memory itself: one launch in place of two uploads, two events
+// and a download in a row, whose latencies a caller that waits for each mask
+// pays in full (a frame, copied against in place: 320x240 M = 3 33.0 and 19.6 us,
+// FP16/BF16 1280x720 M = 5 73.2 and 45.6, FP32 1920x1080 M = 5 141 and 81,
+// 3840x2160 M = 3 396 and 255).
+static int apply_host_in_place(gmm_ctx *h, const uint8_t *rgb, const uint16_t *depth,
+                               uint32_t *mask) {
+    TraceRange tr("gmm_apply_host");
+    if (!h->ev_host) {
+        const cudaError_t e = cudaEventCreateWithFlags(&h->ev_host, cudaEventDisableTiming);
+        if (e != cudaSuccess)
+            return cuda_fail(&h->sticky, e, "gmm_apply_host");
+    }
+    int rc = launch_apply(h, rgb, depth, mask, nullptr, nullptr);
+    if (rc != GMM_OK)
+        return rc;
+    const cudaError_t e = cudaEventRecord(h->ev_host, h->stream);
+    if (e != cudaSuccess)
+        return cuda_fail(&h->sticky, e, "gmm_apply_host");
+    rc = wait_event(h->ev_host, -1, &h->sticky, "gmm_apply_host");
+    if (rc == GMM_OK)
+        h->done_upto = h->next_ticket++; // a frame takes a ticket on either path
+    return rc;
+}
+
 int gmm_apply_host(gmm_t *h, const uint8_t *rgb8_host, const uint16_t *depth16_host,
                    uint32_t *mask_host) {
+    if (h && h->sticky == cudaSuccess && rgb8_host && depth16_host && mask_host &&
+        h->done_upto + 1 == h->next_ticket) {
+        DeviceGuard g(h->device);
+        if (in_place(h, rgb8_host, depth16_host, mask_host))
+            return apply_host_in_place(h, rgb8_host, depth16_host, mask_host);
+    }
     const long long t = gmm_pipe_submit(h, rgb8_host, depth16_host, mask_host);
     if (t < 0)
         return (int)t;
@@ -757,6 +814,8 @@ int gmm_destroy(gmm_t *h) {
         cudaStreamDestroy(h->s_up);
         cudaStreamDestroy(h->s_down);
     }
+    if (h->ev_host)
+        cudaEventDestroy(h->ev_host);
     cudaFree(h->arena);
     if (h->morph_tmp)
         cudaFree(h->morph_tmp);
