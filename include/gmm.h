@@ -396,26 +396,23 @@ int gmm_pool_set_stream(gmm_pool_t *p, void *cuda_stream);
 
 /* Launch shape of the pooled kernel: threads per block (64..256, a
  * multiple of 32); CTAs per SM of the persistent form (>= 1; its CTAs loop
- * over tiles of tile_pixels pixels, a multiple of the block size), or -1
- * for the flat form (a grid over the launch's pixels in which every warp
+ * over tiles of tile_pixels pixels, a multiple of the block size, or of
+ * fewer where a tick has too few pixels for such tiles to occupy every CTA
+ * evenly), or -1 for the flat form (a grid over the launch's pixels in which every warp
  * takes one chunk of 32 pixels, FP32, or 64, FP16/BF16, and exits;
  * tile_pixels is then unused). 0 keeps the current value (initially: 128
  * threads, as many persistent CTAs as fit, 2048-pixel tiles). */
 int gmm_pool_set_launch(gmm_pool_t *p, int threads, int ctas_per_sm,
                         int tile_pixels);
 
-/* Next-tile prefetch of the FP16/BF16 persistent form (enable = 1, the
- * default; 0 turns it off). With a launch shape whose tiles hold at most two
- * pixels per thread, a CTA takes its next tile when the current one starts
- * (except in the last two waves of a tick's tiles) and prefetches that
- * tile's first pixels' state into L2. Measured on the 64-camera mix: 94-95%
- * of the HBM copy bandwidth instead of 90-91% with the frames in device
- * memory, and no loss with frames read over the host link; but when frames
- * are uploaded on a copy stream beside each tick, the uploads slow down
- * (end to end 29 against 36-40 Gpixel-frames/s) and the online tuner's
- * trial ticks do not show it, so such pipelines should turn it off. It
- * changes no result (bit for bit the same either way) and does nothing for
- * FP32 pools. Applies from the next tick. GMM_EINVAL on a null pool. */
+/* L2 prefetch of the FP16/BF16 persistent form (enable = 1, the default; 0
+ * turns it off): while a warp works on its 32 pixels of a tile it prefetches
+ * the state of its next 32. Measured on 24 cameras of odd sizes: 340 -> 330 us
+ * per tick. It competes with frames uploaded on a copy stream beside each
+ * tick, so such pipelines should turn it off. It changes no result (bit for
+ * bit the same either way) and does nothing for FP32 pools (which always
+ * prefetch) or for ticks with cameras that use the options. Applies from the
+ * next tick. GMM_EINVAL on a null pool. */
 int gmm_pool_set_prefetch(gmm_pool_t *p, int enable);
 
 /* Time each candidate launch shape on the current submissions (the state is

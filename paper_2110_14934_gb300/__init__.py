@@ -436,7 +436,7 @@ class Pool:
         _check(load_library().gmm_pool_use_graph(self._p, int(bool(enable))))
 
     def set_prefetch(self, enable=True) -> None:
-        """FP16/BF16 next-tile L2 prefetch (on by default); turn it off when
+        """FP16/BF16 L2 prefetch (on by default); turn it off when
         frames are uploaded on a copy stream beside every tick."""
         _check(load_library().gmm_pool_set_prefetch(self._p, int(bool(enable))))
 

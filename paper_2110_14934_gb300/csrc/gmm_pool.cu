@@ -106,7 +106,7 @@ struct gmm_pool {
     bool staged_used[kStaging] = {};
     int buf = 0;
     bool use_graph = false;
-    bool prefetch = true; // FP16/BF16: next-tile L2 prefetch in the persistent form
+    bool prefetch = true; // FP16/BF16: L2 prefetch in the persistent form
     cudaGraphExec_t gexec[kStaging] = {};
     GraphSig gsig[kStaging];
     Tuning tune;
@@ -288,13 +288,33 @@ static cudaError_t launch_tick(gmm_pool *p, int b, int n_launch, bool all_varian
     return e;
 }
 
+// Tile size of a tick of the persistent form: the pool's, or less where that
+// would leave too few tiles or an uneven last wave. share: a CTA's share of the
+// tick's pixels. Large ticks: a sixteenth of it, so the CTAs end together (24
+// FP16/BF16 cameras, 17 M pixels: 328 us with 2048-pixel tiles, 318 with 896).
+// Small ones: about four pixels per thread, in as many equal parts as the
+// share holds, at least one (4 cameras, 2.9 M pixels: 79 us with 2048-pixel
+// tiles, which only reach half of the CTAs, 52 with 512). A multiple of the
+// block size.
+static int tick_tile(const gmm_pool *p, int64_t pixels, int blocks) {
+    const int64_t threads = p->threads, four = 4 * threads;
+    const int64_t share = (pixels + blocks - 1) / blocks;
+    int64_t tile = share / 16 / threads * threads;
+    if (tile < four) {
+        const int64_t parts = (share + four / 2) / four;
+        tile = parts > 1 ? (share + parts - 1) / parts : share;
+        tile = (tile + threads - 1) / threads * threads;
+    }
+    return tile < p->tile_pixels ? (int)tile : p->tile_pixels;
+}
+
 // One tick over the submitted cameras. clear: drop the submissions and mark
 // the cameras initialised afterwards (false while autotuning).
 static int pool_tick_impl(gmm_pool *p, bool clear) {
-    int n_jobs = 0;
+    int64_t pixels = 0;
     for (const PoolCam &c : p->cams)
-        n_jobs += (c.used && c.submitted) ? 1 : 0;
-    if (n_jobs == 0)
+        pixels += (c.used && c.submitted) ? c.L.n_pad : 0;
+    if (pixels == 0)
         return GMM_OK;
     // An online-tuning trial sets its launch shape first: the tile tables
     // below depend on the tile size.
@@ -317,7 +337,8 @@ static int pool_tick_impl(gmm_pool *p, bool clear) {
     }
     // The launches' arguments: up to kPoolViews cameras each.
     // tiles, or in the flat form one chunk per warp
-    const int unit = p->ctas_per_sm < 0 ? chunk_pixels(p->prec) : p->tile_pixels;
+    const int unit = p->ctas_per_sm < 0 ? chunk_pixels(p->prec)
+                                        : tick_tile(p, pixels, blocks_for(p));
     int *cur = p->d_counters + p->parity * p->kmax;
     int *next = p->d_counters + (1 - p->parity) * p->kmax;
     int li = 0, j = 0;

@@ -22,30 +22,33 @@ namespace {
 // the views are read from the constant bank where they are used and hold no
 // registers across a pixel's arithmetic.
 __constant__ PoolArgs c_pool;
-template <int M, int PREC, int V>
+
+// kPF: the state of a warp's next 32 pixels of the tile moves towards L2 while
+// it works on the current ones (64 FP32 cameras 1361 -> 1279 us, 24 FP16/BF16
+// ones of odd sizes 340 -> 330; two steps ahead 1338 and 337, with the List-1
+// bytes 1309 and 333; with the frame values a step ahead in registers, which
+// spill, 1315 and 331).
+template <int M, int PREC, int V, bool kPF>
 __device__ __forceinline__ void pool_tile(const CamView &cv, int64_t p0, int64_t p1) {
     for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-        // p1 - p0 is a multiple of 32 and blockDim too: warps stay whole. The
-        // state of the CTA's next pixels moves towards L2 meanwhile (64 FP32
-        // cameras 1361 -> 1279 us, 24 FP16/BF16 ones of odd sizes 340 -> 330;
-        // two steps ahead 1338 and 337, with the List-1 bytes 1309 and 333).
-        if (p + blockDim.x < p1)
+        // p1 - p0 is a multiple of 32 and blockDim too: warps stay whole.
+        if (kPF && p + blockDim.x < p1)
             prefetch_pixels<M, PREC, V>(cv, p + blockDim.x);
         const uint32_t bits = process_pixel<M, PREC, V>(cv, p);
         write_mask_words(cv, p >> 5, bits);
     }
 }
 
-template <int M, int PREC, bool kAll>
+template <int M, int PREC, bool kAll, bool kPF>
 __device__ __forceinline__ void pool_tile_v(const CamView &cv, int64_t p0, int64_t p1) {
     if (!kAll) {
-        pool_tile<M, PREC, 0>(cv, p0, p1);
+        pool_tile<M, PREC, 0, kPF>(cv, p0, p1);
         return;
     }
     switch (gmmhost::view_variant(cv)) {
-    case 0: pool_tile<M, PREC, 0>(cv, p0, p1); break;
-    case 1: pool_tile<M, PREC, 1>(cv, p0, p1); break;
-    default: pool_tile<M, PREC, 2>(cv, p0, p1); break;
+    case 0: pool_tile<M, PREC, 0, kPF>(cv, p0, p1); break;
+    case 1: pool_tile<M, PREC, 1, kPF>(cv, p0, p1); break;
+    default: pool_tile<M, PREC, 2, kPF>(cv, p0, p1); break;
     }
 }
 
@@ -64,123 +67,42 @@ __device__ __forceinline__ int tile_job(const PoolArgs &a, int64_t t) {
     return lo;
 }
 
-// Bulk prefetch of [p, p + bytes) into L2 (a hint: nothing waits for it);
-// p and bytes multiples of 16.
-__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
-// L2 bytes the prefetched next tiles of all CTAs may hold together (state
-// and List-1 bytes): each CTA prefetches the first pixels of its next tile,
-// as many whole 256-pixel state tiles as its share of this budget holds (at
-// least one). Past about this much, prefetched lines are evicted before their
-// loads arrive and the data crosses HBM twice.
-constexpr int64_t kPrefetchBudget = 16ll << 20;
-
-// Prefetch the state and List-1 bytes of the first pixels of tile t (camera
-// job) into L2: of each 256-pixel state tile the planes that every tick reads,
-// one contiguous block at its head (the camera's allocation holds every state
-// tile up to n_tiles); the List-1 bytes start at a multiple of 32 and number a
-// multiple of 32.
-__device__ __forceinline__ void prefetch_tile(const PoolArgs &a, int64_t t, int job) {
-    const CamView &v = a.views[job];
-    const int64_t tile_bytes = (int64_t)kFields * v.M * kTile * 2;
-    const uint32_t head = (uint32_t)(2 * v.M + 2) * kTile * 4;
-    const int64_t share = kPrefetchBudget / gridDim.x / (head + kTile);
-    const int64_t q0 = (t - a.tile_begin[job]) * a.tile_pixels;
-    const int64_t s0 = q0 / kTile;
-    const int64_t q1 = min(min(q0 + (int64_t)a.tile_pixels, v.n_pad),
-                           (s0 + max(share, (int64_t)1)) * kTile);
-    const int64_t s1 = (q1 + kTile - 1) / kTile;
-    for (int64_t s = s0; s < s1; ++s)
-        prefetch_l2(static_cast<const char *>(v.planes) + s * tile_bytes, head);
-    prefetch_l2(v.fusion + q0, (uint32_t)(q1 - q0));
-}
-
-// Take the CTA's next tile from the counter into slot `slot` (thread 0),
-// prefetching its first pixels' state when asked.
-__device__ __forceinline__ void take_next(const PoolArgs &a, int64_t *s_tile, int *s_job,
-                                          int slot, bool prefetch) {
-    const int64_t tn = atomicAdd(a.counter, 1);
-    const int jn = tile_job(a, tn);
-    s_tile[slot] = tn;
-    s_job[slot] = jn;
-    if (prefetch && tn < a.n_tiles)
-        prefetch_tile(a, tn, jn);
-}
-
 // kAll: tiles may come from cameras that use the options or the
 // augmentation alternative (launched only when such a camera is in the tick).
 // Registers: 64 (32 resident warps per SM; FP16/BF16 at 48 and 40 warps spills
 // and measures 331 us against 322 on 24 cameras of odd sizes), the FP32
-// instance that also handles the options 80.
-// FP32 state, the instance that also handles the options, and FP16/BF16
-// pools that turned the prefetch off (kPF = false): thread 0 takes a tile
-// from the counter and publishes it between two barriers. Otherwise, in
-// FP16/BF16 state (kPrefetch): a CTA's current and next tile (and camera) sit
-// in alternate slots; thread 0 takes the next tile at the end of the current
-// one, or, for tiles of at most two pixels per thread while at least two
-// waves of tiles remain beyond the current one, at its start, and then
-// prefetches the next tile's first pixels' state into L2, so those loads
-// find the data on chip (with FP16/BF16 state the bytes a warp keeps in
-// flight in its registers do not cover HBM latency). Taken early near the
-// end of the worklist, a CTA would hold two tiles while others run out of
-// work; with more pixels per thread per tile, and with FP32 state
-// (HBM-bound), prefetching measured slower. One barrier per tile; slot k ^ 1
-// is written only after the barrier that ended the tile at whose start every
-// thread last read it.
-template <int PREC, bool kAll, bool kPF = true>
+// instance that also handles the options 80. Thread 0 takes a tile from the
+// counter and publishes it between two barriers. (Taking the next tile at the
+// start of the current one and prefetching its head measured 913 us against
+// 842 on 64 FP16/BF16 cameras, each at its best launch shape, now that a tile
+// prefetches within itself.)
+template <int PREC, bool kAll, bool kPF>
 __global__ void __launch_bounds__(256, PREC == 0 && kAll ? 3 : 4) k_pool_tick() {
-    constexpr bool kPrefetch = PREC != 0 && !kAll && kPF;
     const PoolArgs &a = c_pool;
-    __shared__ int64_t s_tile[2];
-    __shared__ int s_job[2];
+    __shared__ int64_t s_tile;
+    __shared__ int s_job;
     if (blockIdx.x == 0) // the next tick's counters (their last users have finished)
         for (int i = threadIdx.x; i < a.n_reset; i += blockDim.x)
             a.reset[i] = 0;
-    if constexpr (!kPrefetch) {
-        for (;;) { // take a tile, publish it, read it, barrier (slot 0 is rewritten)
-            if (threadIdx.x == 0)
-                take_next(a, s_tile, s_job, 0, false);
-            __syncthreads();
-            const int64_t t = s_tile[0];
-            const int job = s_job[0];
-            __syncthreads();
-            if (t >= a.n_tiles)
-                return;
-            const CamView &cv = a.views[job];
-            const int64_t p0 = (t - a.tile_begin[job]) * a.tile_pixels;
-            const int64_t p1 = min(p0 + (int64_t)a.tile_pixels, cv.n_pad);
-            switch (cv.M) {
-            case 3: pool_tile_v<3, PREC, kAll>(cv, p0, p1); break;
-            case 4: pool_tile_v<4, PREC, kAll>(cv, p0, p1); break;
-            default: pool_tile_v<5, PREC, kAll>(cv, p0, p1); break;
-            }
+    for (;;) {
+        if (threadIdx.x == 0) {
+            s_tile = atomicAdd(a.counter, 1);
+            s_job = tile_job(a, s_tile);
         }
-    }
-    if (threadIdx.x == 0)
-        take_next(a, s_tile, s_job, 0, false);
-    __syncthreads();
-    for (int k = 0;; k ^= 1) {
-        const int64_t t = s_tile[k];
-        const int job = s_job[k];
+        __syncthreads();
+        const int64_t t = s_tile;
+        const int job = s_job;
+        __syncthreads();
         if (t >= a.n_tiles)
             return;
-        const bool early = a.tile_pixels <= 2 * (int)blockDim.x &&
-                           t + 2 * (int64_t)gridDim.x < a.n_tiles;
-        if (early && threadIdx.x == 0)
-            take_next(a, s_tile, s_job, k ^ 1, true);
         const CamView &cv = a.views[job];
         const int64_t p0 = (t - a.tile_begin[job]) * a.tile_pixels;
         const int64_t p1 = min(p0 + (int64_t)a.tile_pixels, cv.n_pad);
         switch (cv.M) {
-        case 3: pool_tile_v<3, PREC, kAll>(cv, p0, p1); break;
-        case 4: pool_tile_v<4, PREC, kAll>(cv, p0, p1); break;
-        default: pool_tile_v<5, PREC, kAll>(cv, p0, p1); break;
+        case 3: pool_tile_v<3, PREC, kAll, kPF>(cv, p0, p1); break;
+        case 4: pool_tile_v<4, PREC, kAll, kPF>(cv, p0, p1); break;
+        default: pool_tile_v<5, PREC, kAll, kPF>(cv, p0, p1); break;
         }
-        if (!early && threadIdx.x == 0)
-            take_next(a, s_tile, s_job, k ^ 1, false);
-        __syncthreads();
     }
 }
 
@@ -321,23 +243,23 @@ cudaError_t launch_pool_tick_impl(const PoolArgs *args_host, int threads, int bl
         else
             launch_flat<1, true>(m, blocks, threads, s);
     } else if (prec == 0 && !all_variants)
-        k_pool_tick<0, false><<<blocks, threads, 0, s>>>();
+        k_pool_tick<0, false, true><<<blocks, threads, 0, s>>>();
     else if (prec == 0)
-        k_pool_tick<0, true><<<blocks, threads, 0, s>>>();
+        k_pool_tick<0, true, true><<<blocks, threads, 0, s>>>();
     else if (!all_variants && prefetch)
-        k_pool_tick<1, false><<<blocks, threads, 0, s>>>();
+        k_pool_tick<1, false, true><<<blocks, threads, 0, s>>>();
     else if (!all_variants)
         k_pool_tick<1, false, false><<<blocks, threads, 0, s>>>();
     else
-        k_pool_tick<1, true><<<blocks, threads, 0, s>>>();
+        k_pool_tick<1, true, false><<<blocks, threads, 0, s>>>();
     return cudaGetLastError();
 }
 
 int pool_max_ctas_per_sm(int prec, int threads) {
     int n = 0;
     cudaError_t e = prec == 0
-        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_pool_tick<0, false>, threads, 0)
-        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_pool_tick<1, false>, threads, 0);
+        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_pool_tick<0, false, true>, threads, 0)
+        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_pool_tick<1, false, true>, threads, 0);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return 1;

@@ -283,13 +283,9 @@ extern "C" {
 double gmm_server_now(void) { return clock_s(); }
 
 // Launch shape of the engine's pool. FP16/BF16 state in the zero-copy mode:
-// 256-thread CTAs (as many as fit) over 512-pixel tiles, whose CTAs prefetch
-// their next tile (the pool tuner's choice on the 64-camera mix; it also
-// splits small ticks into more tiles). Measured on the 256-camera schedule:
-// p50 0.114 -> 0.106 ms, p99 0.26 -> 0.21 ms, the genlocked rig's p50
-// 0.68 -> 0.47 ms. Otherwise the pool's default (128 threads, 2048-pixel
-// tiles, no early take): the copy mode uploads frames beside the running
-// tick, and its latency tail grew with the other shape.
+// 256-thread CTAs (as many as fit) over tiles of at most 512 pixels, a little
+// faster than the pool's default with frames read over the host link (4 cameras
+// of 1280x720 159 us a tick against 161). Otherwise the pool's default.
 static void set_pool_shape(gmm_server *s) {
     if (s->prec == GMM_PREC_F16 && s->transfer == GMM_SERVE_ZERO_COPY)
         gmm_pool_set_launch(s->pool, 256, 0, 512);
