@@ -44,8 +44,7 @@
  *    pixel x = 32*c + i (least significant bit first); bits for x >= W are 0.
  *  - A CUDA failure is sticky on the handle: later calls return GMM_ECUDA.
  *  - Threads: a handle or a pool is used by one thread at a time (calls on
- *    different handles and pools may run concurrently, and pools on one
- *    device share their launch-argument bank safely); the gmm_server_*
+ *    different handles and pools may run concurrently); the gmm_server_*
  *    calls other than gmm_server_destroy may be made from any thread.
  *    Device work is ordered on the object's stream.
  */
@@ -426,8 +425,8 @@ int gmm_pool_autotune(gmm_pool_t *p, int iters, int *threads,
 /* Online tuning of the launch shape on real ticks: the next
  * ticks_per_shape x (number of candidates) calls of gmm_pool_tick each run
  * one candidate shape (block size 64/128/256; the persistent form at full or
- * half residency with tiles of 256/512/1024/2048/8192 pixels; round-robin, CUDA
- * graphs off meanwhile; the flat form is chosen only explicitly). Each such tick is timed on the
+ * half residency with tiles of 256/512/1024/2048/8192 pixels; round-robin;
+ * the flat form is chosen only explicitly). Each such tick is timed on the
  * pool's stream from its start to the start of the next tick (the tick
  * period, so whatever the tick's kernel delays among the work queued before
  * the next tick, such as uploads of the next frames, counts against its
@@ -435,7 +434,7 @@ int gmm_pool_autotune(gmm_pool_t *p, int iters, int *threads,
  * periods run a second round of 2 x ticks_per_shape ticks each (ticks
  * between the rounds, until the first round's timings are read, keep the
  * last trial's shape), and the one with the lowest median period in that
- * round is kept and graph use restored. The ticks do their
+ * round is kept. The ticks do their
  * normal work, so nothing is snapshotted. gmm_pool_set_launch during tuning
  * is overridden. */
 int gmm_pool_autotune_online(gmm_pool_t *p, int ticks_per_shape);
@@ -445,10 +444,9 @@ int gmm_pool_autotune_online(gmm_pool_t *p, int ticks_per_shape);
  * the non-NULL outputs. */
 int gmm_pool_tuning(gmm_pool_t *p, int *threads, int *ctas_per_sm, int *tile_pixels);
 
-/* Run the pool's tick as a CUDA graph (enable = 1): the graph of the tick's
- * launches is built once and replayed every tick, its kernel nodes updated
- * with the tick's cameras; it is rebuilt when the number of launches (one
- * per 128 cameras), the launch shape or the kernel instance changes. */
+/* Accepted in either state and without effect: a tick is one kernel launch
+ * (per 128 cameras) whose arguments travel with it, so a CUDA graph of it
+ * would hold just that launch. */
 int gmm_pool_use_graph(gmm_pool_t *p, int enable);
 
 /* As gmm_state_get, for camera cam. */

@@ -55,8 +55,7 @@ cudaError_t launch_morph_open3(const uint32_t *in, uint32_t *out, int H, int W,
 // [tile_begin[j], tile_begin[j+1]) of camera views[j], tile_pixels pixels
 // each (the last one of a camera ragged). A launch handles up to kPoolViews
 // cameras (a tick with more is split into several launches); its PoolArgs
-// are copied into the kernel's constant memory on the stream right before
-// it. *counter must be zero at launch; the launch zeroes the n_reset
+// are the kernel's parameters. *counter must be zero at launch; the launch zeroes the n_reset
 // counters at reset (the next tick's).
 constexpr int kPoolViews = 128;
 struct PoolArgs {
@@ -69,26 +68,18 @@ struct PoolArgs {
     int tile_pixels;
     int64_t n_tiles;
 };
-static_assert(sizeof(PoolArgs) <= 32768, "one launch's arguments fit half the constant bank");
+static_assert(sizeof(PoolArgs) <= 32764, "one launch's arguments fit the kernel parameters");
 
-// Upload *args_host (page-locked for an asynchronous copy) to the kernel's
-// constant memory and launch the pool kernel; all_variants: the instance
+// Launch the pool kernel; all_variants: the instance
 // that also handles the options and the augmentation alternative; flat: the
 // non-persistent form (tile_begin and n_tiles count one chunk per warp:
 // 32 pixels in FP32, 64 in FP16/BF16; blocks covers every chunk); m: the M
 // every camera of the launch has (a kernel specialised to it), or 0;
 // prefetch: the FP16/BF16 persistent instance that prefetches each warp's next
 // pixels into L2 (else the one that does not).
-cudaError_t launch_pool_tick_impl(const PoolArgs *args_host, int threads, int blocks, int prec,
+cudaError_t launch_pool_tick_impl(const PoolArgs &args, int threads, int blocks, int prec,
                                   bool all_variants, bool flat, int m, bool prefetch,
                                   cudaStream_t s);
-
-// The constant-memory argument bank is shared by every pool on a device:
-// enqueue uploads and launches between acquire (takes the device's lock and
-// orders stream s after the bank's previous user) and release (records s as
-// the last user, drops the lock). Not needed while capturing a graph.
-cudaError_t pool_bank_acquire(int device, cudaStream_t s);
-cudaError_t pool_bank_release(int device, cudaStream_t s);
 
 // process_pixel variant a camera needs: 0 default, 1 learning-rate/variance
 // options, 2 augmentation alternative.

@@ -1,6 +1,6 @@
 // Multi-camera pool: resident per-camera models, one persistent launch per
-// tick over every camera with a submitted frame, optional CUDA-graph replay
-// of the tick, and an autotuner for the launch shape.
+// tick over every camera with a submitted frame, and an autotuner for the
+// launch shape.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -32,22 +32,6 @@ struct PoolCam {
     uint32_t *mask = nullptr, *fgr = nullptr, *fgd = nullptr;
 };
 
-// What a captured graph depends on. The views and tile tables are read at
-// replay from the page-locked staging buffer the graph was captured with.
-struct GraphSig {
-    int n_launch = -1, threads = 0;
-    std::vector<int> blocks; // per launch
-    std::vector<int> m; // per launch: the M its cameras share (flat form), else 0
-    bool all_variants = false, flat = false, prefetch = true;
-    bool operator==(const GraphSig &o) const {
-        return n_launch == o.n_launch && threads == o.threads && blocks == o.blocks &&
-               m == o.m && all_variants == o.all_variants && flat == o.flat &&
-               prefetch == o.prefetch;
-    }
-};
-
-constexpr int kStaging = 2; // page-locked argument buffers, used alternately
-
 // ctas < 0: the flat (non-persistent) form; tile is then its chunk size.
 struct Shape {
     int threads, ctas, tile;
@@ -71,7 +55,6 @@ struct Trial {
 constexpr int kFinalists = 4;
 struct Tuning {
     bool active = false;
-    bool saved_graph = false;
     bool final_round = false;
     int per_shape = 0, issued = 0;
     std::vector<Shape> cands;
@@ -91,7 +74,6 @@ struct gmm_pool {
     int prec = 0, max_cams = 0, device = 0;
     std::vector<PoolCam> cams;
     cudaStream_t stream = nullptr;
-    cudaStream_t cap_stream = nullptr; // graph capture (the legacy stream cannot capture)
     cudaMemPool_t mempool = nullptr;   // cameras' state; keeps freed memory mapped
     cudaError_t sticky = cudaSuccess;
     int threads = 128, ctas_per_sm = 0, tile_pixels = 2048; // ctas_per_sm < 0: flat form
@@ -100,28 +82,12 @@ struct gmm_pool {
     int *d_counters = nullptr;
     int kmax = 1, parity = 0; // kmax: launches a tick may take
     std::vector<int> launch_m; // per launch: the M its cameras share (flat form), else 0
-    // Launch arguments (kmax per tick) in page-locked memory, two buffers.
-    gmmhost::PoolArgs *h_args[kStaging] = {};
-    cudaEvent_t ev_staged[kStaging] = {};
-    bool staged_used[kStaging] = {};
-    int buf = 0;
-    bool use_graph = false;
+    std::vector<gmmhost::PoolArgs> args; // of a tick's launches (kmax)
     bool prefetch = true; // FP16/BF16: L2 prefetch in the persistent form
-    cudaGraphExec_t gexec[kStaging] = {};
-    GraphSig gsig[kStaging];
     Tuning tune;
     int occupancy[9] = {};  // resident pool CTAs per SM, by block size / 32
     int sms = 0;
 };
-
-static void destroy_graphs(gmm_pool *p) {
-    for (int b = 0; b < kStaging; ++b) {
-        if (p->gexec[b])
-            cudaGraphExecDestroy(p->gexec[b]);
-        p->gexec[b] = nullptr;
-        p->gsig[b] = GraphSig();
-    }
-}
 
 // Resident CTAs per SM of the pool kernel for a block size (queried once per
 // block size) times the SM count (queried once).
@@ -217,93 +183,40 @@ static int tuning_poll(gmm_pool *p, bool block) {
     p->threads = tu.cands[best].threads;
     p->ctas_per_sm = tu.cands[best].ctas;
     p->tile_pixels = tu.cands[best].tile;
-    p->use_graph = tu.saved_graph;
     tu.active = false;
     return GMM_OK;
 }
 
-// Enqueue the tick's launches (argument upload + persistent kernel each)
-// from staging buffer b.
-static cudaError_t enqueue_body(gmm_pool *p, cudaStream_t s, int b, const GraphSig &sig) {
-    cudaError_t e = cudaSuccess;
-    for (int li = 0; li < sig.n_launch && e == cudaSuccess; ++li)
-        e = gmmhost::launch_pool_tick_impl(&p->h_args[b][li], sig.threads, sig.blocks[li],
-                                           p->prec, sig.all_variants, sig.flat, sig.m[li],
-                                           sig.prefetch, s);
-    return e;
-}
-
-// Launch the tick, directly or by replaying the graph captured for staging
-// buffer b (captured again when its shape changed).
-static cudaError_t launch_tick(gmm_pool *p, int b, int n_launch, bool all_variants) {
-    GraphSig sig;
-    sig.n_launch = n_launch;
-    sig.threads = p->threads;
-    sig.all_variants = all_variants;
-    sig.flat = p->ctas_per_sm < 0;
-    sig.prefetch = p->prefetch;
+// Launch the tick's n_launch launches.
+static cudaError_t launch_tick(gmm_pool *p, int n_launch, bool all_variants) {
+    const bool flat = p->ctas_per_sm < 0;
     const int warps = p->threads / 32;
-    for (int li = 0; li < n_launch; ++li) { // flat: one warp per chunk
-        sig.blocks.push_back(sig.flat ? (int)((p->h_args[b][li].n_tiles + warps - 1) / warps)
-                                      : blocks_for(p));
-        sig.m.push_back(p->launch_m[li]);
-    }
-    if (!p->use_graph) {
-        cudaError_t e = gmmhost::pool_bank_acquire(p->device, p->stream);
-        if (e != cudaSuccess)
-            return e;
-        e = enqueue_body(p, p->stream, b, sig);
-        const cudaError_t er = gmmhost::pool_bank_release(p->device, p->stream);
-        return e != cudaSuccess ? e : er;
-    }
     cudaError_t e = cudaSuccess;
-    if (!(p->gexec[b] && p->gsig[b] == sig)) {
-        if (p->gexec[b])
-            cudaGraphExecDestroy(p->gexec[b]);
-        p->gexec[b] = nullptr;
-        p->gsig[b] = GraphSig();
-        cudaGraph_t g = nullptr;
-        e = cudaStreamBeginCapture(p->cap_stream, cudaStreamCaptureModeThreadLocal);
-        if (e == cudaSuccess) {
-            const cudaError_t eb = enqueue_body(p, p->cap_stream, b, sig);
-            e = cudaStreamEndCapture(p->cap_stream, &g);
-            if (eb != cudaSuccess)
-                e = eb;
-        }
-        if (e == cudaSuccess)
-            e = cudaGraphInstantiate(&p->gexec[b], g, 0);
-        if (g)
-            cudaGraphDestroy(g);
-        if (e == cudaSuccess)
-            p->gsig[b] = sig;
-    }
-    if (e == cudaSuccess)
-        e = gmmhost::pool_bank_acquire(p->device, p->stream);
-    if (e == cudaSuccess) {
-        e = cudaGraphLaunch(p->gexec[b], p->stream);
-        const cudaError_t er = gmmhost::pool_bank_release(p->device, p->stream);
-        if (e == cudaSuccess)
-            e = er;
+    for (int li = 0; li < n_launch && e == cudaSuccess; ++li) {
+        const gmmhost::PoolArgs &a = p->args[li];
+        const int blocks = flat ? (int)((a.n_tiles + warps - 1) / warps) : blocks_for(p);
+        e = gmmhost::launch_pool_tick_impl(a, p->threads, blocks, p->prec, all_variants, flat,
+                                           p->launch_m[li], p->prefetch, p->stream);
     }
     return e;
 }
 
 // Tile size of a tick of the persistent form: the pool's, or less where that
 // would leave too few tiles or an uneven last wave. share: a CTA's share of the
-// tick's pixels. Large ticks: a sixteenth of it, so the CTAs end together (24
-// FP16/BF16 cameras, 17 M pixels: 328 us with 2048-pixel tiles, 318 with 896).
-// Small ones: about four pixels per thread, in as many equal parts as the
-// share holds, at least one (4 cameras, 2.9 M pixels: 79 us with 2048-pixel
-// tiles, which only reach half of the CTAs, 52 with 512). A multiple of the
-// block size.
+// tick's pixels. Large ticks: a sixteenth of it, so the CTAs end together.
+// Smaller ones: about four pixels per thread, in as many equal parts as the
+// share holds. A multiple of the block size. (us per tick, tiles of 256, 512,
+// 896, 2048 pixels: 40 cameras of odd sizes, 29 M pixels, FP16/BF16 477, 442,
+// 429, 427, and 1280 426; 24 cameras, 17 M pixels, FP16/BF16 332, 311, 304, 308,
+// FP32 452, 434, 435, 449; 9 cameras, 6.8 M pixels, FP16/BF16 134, 126, 125,
+// 128; 4 cameras, 3.4 M pixels, FP32 102, 103, 107, 119.)
 static int tick_tile(const gmm_pool *p, int64_t pixels, int blocks) {
     const int64_t threads = p->threads, four = 4 * threads;
     const int64_t share = (pixels + blocks - 1) / blocks;
     int64_t tile = share / 16 / threads * threads;
     if (tile < four) {
-        const int64_t parts = (share + four / 2) / four;
-        tile = parts > 1 ? (share + parts - 1) / parts : share;
-        tile = (tile + threads - 1) / threads * threads;
+        const int64_t parts = (share + four - 1) / four;
+        tile = ((share + parts - 1) / parts + threads - 1) / threads * threads;
     }
     return tile < p->tile_pixels ? (int)tile : p->tile_pixels;
 }
@@ -328,13 +241,6 @@ static int pool_tick_impl(gmm_pool *p, bool clear) {
         p->ctas_per_sm = tu.cands[tr.cand].ctas;
         p->tile_pixels = tu.cands[tr.cand].tile;
     }
-    const int b = p->buf;
-    if (p->staged_used[b]) {
-        // The uploads that last read this staging buffer must have run.
-        const int rc = wait_event(p->ev_staged[b], 60000, &p->sticky, "gmm_pool_tick staging");
-        if (rc != GMM_OK)
-            return rc;
-    }
     // The launches' arguments: up to kPoolViews cameras each.
     // tiles, or in the flat form one chunk per warp
     const int unit = p->ctas_per_sm < 0 ? chunk_pixels(p->prec)
@@ -347,7 +253,7 @@ static int pool_tick_impl(gmm_pool *p, bool clear) {
     const bool flat = p->ctas_per_sm < 0;
     int group_m = 0; // flat form: the launch's cameras share M (a kernel per M)
     auto close_launch = [&]() {
-        gmmhost::PoolArgs &a = p->h_args[b][li];
+        gmmhost::PoolArgs &a = p->args[li];
         p->launch_m[li] = group_m;
         a.tile_begin[j] = tiles;
         a.n_jobs = j;
@@ -370,7 +276,7 @@ static int pool_tick_impl(gmm_pool *p, bool clear) {
         for (PoolCam &c : p->cams) {
             if (!(c.used && c.submitted) || c.cfg.M != m)
                 continue;
-            gmmhost::PoolArgs &a = p->h_args[b][li];
+            gmmhost::PoolArgs &a = p->args[li];
             a.views[j] = make_view(c.cfg, c.L, c.arena, c.rgb, c.depth, c.mask, c.fgr, c.fgd,
                                    c.initialized ? 0 : 1, c.ticks);
             all_variants = all_variants || gmmhost::view_variant(a.views[j]) != 0;
@@ -407,13 +313,9 @@ static int pool_tick_impl(gmm_pool *p, bool clear) {
         tu.open = tr;
         ++tu.issued;
     }
-    e = launch_tick(p, b, n_launch, all_variants);
-    if (e == cudaSuccess)
-        e = cudaEventRecord(p->ev_staged[b], p->stream);
+    e = launch_tick(p, n_launch, all_variants);
     if (e != cudaSuccess)
         return cuda_fail(&p->sticky, e, "gmm_pool_tick");
-    p->staged_used[b] = true;
-    p->buf = (b + 1) % kStaging;
     p->parity ^= 1;
     if (clear) {
         for (PoolCam &c : p->cams) {
@@ -454,14 +356,8 @@ gmm_pool_t *gmm_pool_create(size_t budget_bytes, int precision, int max_cams) {
     // one launch per kPoolViews cameras, plus one per M group in the flat form
     p->kmax = (max_cams + gmmhost::kPoolViews - 1) / gmmhost::kPoolViews + 2;
     p->launch_m.assign((size_t)p->kmax, 0);
+    p->args.resize((size_t)p->kmax);
     cudaError_t e = cudaGetDevice(&p->device);
-    for (int b = 0; b < kStaging && e == cudaSuccess; ++b) {
-        e = cudaMallocHost(&p->h_args[b], sizeof(gmmhost::PoolArgs) * (size_t)p->kmax);
-        if (e == cudaSuccess)
-            e = cudaEventCreateWithFlags(&p->ev_staged[b], cudaEventDisableTiming);
-    }
-    if (e == cudaSuccess)
-        e = cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess)
         e = cudaMalloc(&p->d_counters, sizeof(int) * 2 * (size_t)p->kmax);
     if (e == cudaSuccess)
@@ -605,8 +501,6 @@ int gmm_pool_tick(gmm_pool_t *p) {
 int gmm_pool_set_stream(gmm_pool_t *p, void *cuda_stream) {
     if (!p)
         return fail(GMM_EINVAL, "gmm_pool_set_stream: null pool");
-    if (p->stream != static_cast<cudaStream_t>(cuda_stream))
-        destroy_graphs(p);
     p->stream = static_cast<cudaStream_t>(cuda_stream);
     return GMM_OK;
 }
@@ -640,13 +534,7 @@ int gmm_pool_set_prefetch(gmm_pool_t *p, int enable) {
 int gmm_pool_use_graph(gmm_pool_t *p, int enable) {
     if (!p)
         return fail(GMM_EINVAL, "gmm_pool_use_graph: null pool");
-    if (p->tune.active) { // applies once online tuning has finished
-        p->tune.saved_graph = enable != 0;
-        return GMM_OK;
-    }
-    p->use_graph = enable != 0;
-    if (!p->use_graph)
-        destroy_graphs(p);
+    (void)enable; // a tick is one launch per 128 cameras and nothing else
     return GMM_OK;
 }
 
@@ -669,8 +557,6 @@ int gmm_pool_autotune_online(gmm_pool_t *p, int ticks_per_shape) {
     tu.per_shape = ticks_per_shape;
     tu.issued = 0;
     tu.final_round = false;
-    tu.saved_graph = p->use_graph;
-    p->use_graph = false; // each trial tick launches directly
     tu.active = true;
     return GMM_OK;
 }
@@ -732,8 +618,6 @@ int gmm_pool_autotune(gmm_pool_t *p, int iters, int *threads_out, int *ctas_out,
     if (e == cudaSuccess)
         e = cudaEventCreate(&t1);
     const int saved_t = p->threads, saved_c = p->ctas_per_sm, saved_tp = p->tile_pixels;
-    const bool saved_graph = p->use_graph;
-    p->use_graph = false;
     int best_t = saved_t, best_c = saved_c, best_tp = saved_tp;
     float best_ms = -1.f;
     const std::vector<Shape> cands = tuning_candidates(p);
@@ -792,7 +676,6 @@ int gmm_pool_autotune(gmm_pool_t *p, int iters, int *threads_out, int *ctas_out,
         cudaEventDestroy(t0);
     if (t1)
         cudaEventDestroy(t1);
-    p->use_graph = saved_graph;
     if (e != cudaSuccess)
         return cuda_fail(&p->sticky, e, "gmm_pool_autotune");
     if (rc != GMM_OK)
@@ -800,7 +683,6 @@ int gmm_pool_autotune(gmm_pool_t *p, int iters, int *threads_out, int *ctas_out,
     p->threads = best_t;
     p->ctas_per_sm = best_c;
     p->tile_pixels = best_tp;
-    destroy_graphs(p);
     if (threads_out)
         *threads_out = best_t;
     if (ctas_out)
@@ -838,7 +720,6 @@ int gmm_pool_destroy(gmm_pool_t *p) {
         return fail(GMM_EINVAL, "gmm_pool_destroy: null pool");
     DeviceGuard g(p->device);
     cudaStreamSynchronize(p->stream);
-    destroy_graphs(p);
     for (Trial &tr : p->tune.pending) {
         cudaEventDestroy(tr.a);
         cudaEventDestroy(tr.b);
@@ -855,14 +736,6 @@ int gmm_pool_destroy(gmm_pool_t *p) {
         cudaMemPoolDestroy(p->mempool);
     if (p->d_counters)
         cudaFree(p->d_counters);
-    if (p->cap_stream)
-        cudaStreamDestroy(p->cap_stream);
-    for (int b = 0; b < kStaging; ++b) {
-        if (p->h_args[b])
-            cudaFreeHost(p->h_args[b]);
-        if (p->ev_staged[b])
-            cudaEventDestroy(p->ev_staged[b]);
-    }
     delete p;
     return GMM_OK;
 }

@@ -1,12 +1,9 @@
 // Multi-camera tick: one launch advances every camera of a pool that has a
 // submitted frame (up to kPoolViews cameras per launch), with the per-pixel
 // arithmetic of the single-camera kernel (gmm_device.cuh), in a persistent
-// form (CTAs loop over tiles) or a flat one (one chunk per warp); and the
-// per-device argument bank their launches share.
+// form (CTAs loop over tiles) or a flat one (one chunk per warp).
 #include <cuda_runtime.h>
 #include <stdint.h>
-
-#include <mutex>
 
 #include "gmm_internal.h"
 
@@ -18,10 +15,17 @@ namespace {
 // ------------------------------------------------------------ kernel
 // CTAs take tiles of the implicit worklist (PoolArgs) from an atomic counter;
 // the camera of a tile is found by binary search over tile_begin. The
-// launch's PoolArgs sit in constant memory (uploaded before each launch), so
-// the views are read from the constant bank where they are used and hold no
-// registers across a pixel's arithmetic.
-__constant__ PoolArgs c_pool;
+// launch's PoolArgs are kernel parameters (24 KB of the 32 KB there may be):
+// the views are read from the constant bank where they are used, hold no
+// registers across a pixel's arithmetic, and reach the device with the launch
+// itself. (Copied into constant memory before each launch, which also had to
+// wait for the last user of that memory, they cost a tick 9 to 12 us: 24
+// FP16/BF16 cameras of odd sizes 311 against 301 us, 4 cameras 52 against 44.)
+// Ticks are programmatic dependents, like the single-camera ones.
+__device__ __forceinline__ void dependent_launch_prologue() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 // kPF: the state of a warp's next 32 pixels of the tile moves towards L2 while
 // it works on the current ones (64 FP32 cameras 1361 -> 1279 us, 24 FP16/BF16
@@ -77,8 +81,9 @@ __device__ __forceinline__ int tile_job(const PoolArgs &a, int64_t t) {
 // 842 on 64 FP16/BF16 cameras, each at its best launch shape, now that a tile
 // prefetches within itself.)
 template <int PREC, bool kAll, bool kPF>
-__global__ void __launch_bounds__(256, PREC == 0 && kAll ? 3 : 4) k_pool_tick() {
-    const PoolArgs &a = c_pool;
+__global__ void __launch_bounds__(256, PREC == 0 && kAll ? 3 : 4) 
+    k_pool_tick(const __grid_constant__ PoolArgs a) {
+    dependent_launch_prologue();
     __shared__ int64_t s_tile;
     __shared__ int s_job;
     if (blockIdx.x == 0) // the next tick's counters (their last users have finished)
@@ -150,8 +155,9 @@ __device__ __forceinline__ void flat_chunk_v(const CamView &cv, int64_t base) {
 // (any M, switched per warp). FP32: no residency hint; FP16/BF16: 64
 // registers, as in the other kernels.
 template <int PREC, bool kAll, int MM>
-__global__ void __launch_bounds__(256, PREC == 0 ? 1 : 4) k_pool_flat() {
-    const PoolArgs &a = c_pool;
+__global__ void __launch_bounds__(256, PREC == 0 ? 1 : 4) 
+    k_pool_flat(const __grid_constant__ PoolArgs a) {
+    dependent_launch_prologue();
     if (blockIdx.x == 0) // the next tick's counters, as the persistent form does
         for (int i = threadIdx.x; i < a.n_reset; i += blockDim.x)
             a.reset[i] = 0;
@@ -180,12 +186,12 @@ __global__ void __launch_bounds__(256, PREC == 0 ? 1 : 4) k_pool_flat() {
 }
 
 template <int PREC, bool kAll>
-void launch_flat(int m, int blocks, int threads, cudaStream_t s) {
+auto flat_kernel(int m) {
     switch (m) {
-    case 3: k_pool_flat<PREC, kAll, 3><<<blocks, threads, 0, s>>>(); break;
-    case 4: k_pool_flat<PREC, kAll, 4><<<blocks, threads, 0, s>>>(); break;
-    case 5: k_pool_flat<PREC, kAll, 5><<<blocks, threads, 0, s>>>(); break;
-    default: k_pool_flat<PREC, kAll, 0><<<blocks, threads, 0, s>>>(); break;
+    case 3: return k_pool_flat<PREC, kAll, 3>;
+    case 4: return k_pool_flat<PREC, kAll, 4>;
+    case 5: return k_pool_flat<PREC, kAll, 5>;
+    default: return k_pool_flat<PREC, kAll, 0>;
     }
 }
 
@@ -193,66 +199,30 @@ void launch_flat(int m, int blocks, int threads, cudaStream_t s) {
 
 namespace gmmhost {
 
-// The argument bank is one per device: launches of different pools (other
-// streams, other threads) take turns through a lock and an event that
-// orders each bank user after the previous one on the GPU.
-namespace {
-struct BankGuard {
-    std::mutex mu;
-    cudaEvent_t last = nullptr;
-};
-BankGuard g_bank[64];
-} // namespace
-
-cudaError_t pool_bank_acquire(int device, cudaStream_t s) {
-    if (device < 0 || device >= 64)
-        return cudaErrorInvalidDevice;
-    BankGuard &g = g_bank[device];
-    g.mu.lock();
-    cudaError_t e = cudaSuccess;
-    if (!g.last)
-        e = cudaEventCreateWithFlags(&g.last, cudaEventDisableTiming);
-    else
-        e = cudaStreamWaitEvent(s, g.last, 0);
-    if (e != cudaSuccess)
-        g.mu.unlock();
-    return e;
-}
-
-cudaError_t pool_bank_release(int device, cudaStream_t s) {
-    BankGuard &g = g_bank[device];
-    const cudaError_t e = cudaEventRecord(g.last, s);
-    g.mu.unlock();
-    return e;
-}
-
-cudaError_t launch_pool_tick_impl(const PoolArgs *args_host, int threads, int blocks, int prec,
+cudaError_t launch_pool_tick_impl(const PoolArgs &args, int threads, int blocks, int prec,
                                   bool all_variants, bool flat, int m, bool prefetch,
                                   cudaStream_t s) {
-    cudaError_t e = cudaMemcpyToSymbolAsync(c_pool, args_host, sizeof(PoolArgs), 0,
-                                            cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess)
-        return e;
-    if (flat) {
-        if (prec == 0 && !all_variants)
-            launch_flat<0, false>(m, blocks, threads, s);
-        else if (prec == 0)
-            launch_flat<0, true>(m, blocks, threads, s);
-        else if (!all_variants)
-            launch_flat<1, false>(m, blocks, threads, s);
-        else
-            launch_flat<1, true>(m, blocks, threads, s);
-    } else if (prec == 0 && !all_variants)
-        k_pool_tick<0, false, true><<<blocks, threads, 0, s>>>();
+    void (*kernel)(PoolArgs);
+    if (flat && prec == 0)
+        kernel = all_variants ? flat_kernel<0, true>(m) : flat_kernel<0, false>(m);
+    else if (flat)
+        kernel = all_variants ? flat_kernel<1, true>(m) : flat_kernel<1, false>(m);
     else if (prec == 0)
-        k_pool_tick<0, true, true><<<blocks, threads, 0, s>>>();
-    else if (!all_variants && prefetch)
-        k_pool_tick<1, false, true><<<blocks, threads, 0, s>>>();
-    else if (!all_variants)
-        k_pool_tick<1, false, false><<<blocks, threads, 0, s>>>();
+        kernel = all_variants ? k_pool_tick<0, true, true> : k_pool_tick<0, false, true>;
+    else if (all_variants)
+        kernel = k_pool_tick<1, true, false>;
     else
-        k_pool_tick<1, true, false><<<blocks, threads, 0, s>>>();
-    return cudaGetLastError();
+        kernel = prefetch ? k_pool_tick<1, false, true> : k_pool_tick<1, false, false>;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args);
 }
 
 int pool_max_ctas_per_sm(int prec, int threads) {
