@@ -5,7 +5,7 @@ and fusion tick on GB300.
 One step = one tick of the whole path (colour mixture, depth mixture, List-1
 fusion, bit-packed mask) over one frame of every camera of the workload. The
 default workload is c2: 64 cameras at mixed resolutions advanced by one
-pooled launch per tick (CUDA graph, online-tuned launch shape), FP32 state.
+pooled launch per tick (online-tuned launch shape), FP32 state.
 The metric is Mpixel-frames/s; the JSON line also carries the HBM roofline
 fraction of the pooled kernel, per-tick latency percentiles, an end-to-end
 figure with host frames and masks, the same cameras one launch per camera
@@ -47,7 +47,7 @@ WORKLOADS = {
                H=1080, W=1920, M=5, kind=1, frames=300, prec=0),
     "c2": dict(name="64 cameras (16 each at 320x240, 640x480, 1280x720, 1920x1080), M from "
                     "{3,5} by seed, FP32 state, 300-frame sequences, one persistent launch per "
-                    "tick (CUDA graph, autotuned launch shape)",
+                    "tick (autotuned launch shape)",
                pool=True, cams_per_res=16, frames=300, prec=0, M=5),
     "c3": dict(name="the 64-camera mix of c2 with FP16 means/variances and BF16 weights (FP32 "
                     "arithmetic), 1000 ticks over 300 resident frames per camera",
@@ -86,7 +86,13 @@ TRAFFIC_RECORDS = {
                        "_flat_f32"),
     ("pool_flat", 1): ("gmm_pool_tick_mixed_cameras.md", ("gmm_device.cuh", "gmm_pool_kernel.cu"),
                        "_flat_f16"),
-    # one-pass captures of the full 64-camera launch (quoted only for that launch)
+    # one-pass captures of the full 64-camera launch: of the workload's scene
+    # (quoted for that launch), and of frames that make every pixel re-rank all
+    # its components (--scene strobe), the tick that has to move the whole state
+    ("pool_scene", 0): ("gmm_pool_tick_mixed_cameras.md", ("gmm_device.cuh", "gmm_pool_kernel.cu"),
+                        "_scene_f32"),
+    ("pool_scene", 1): ("gmm_pool_tick_mixed_cameras.md", ("gmm_device.cuh", "gmm_pool_kernel.cu"),
+                        "_scene_f16"),
     ("pool_full", 0): ("gmm_pool_tick_mixed_cameras.md", ("gmm_device.cuh", "gmm_pool_kernel.cu"),
                        "_full_f32"),
     ("pool_full", 1): ("gmm_pool_tick_mixed_cameras.md", ("gmm_device.cuh", "gmm_pool_kernel.cu"),
@@ -96,11 +102,21 @@ KERNEL_SOURCES = [os.path.join(CSRC, f) for f in TRAFFIC_RECORDS[("tick", 0)][1]
 
 
 def bytes_per_pixel(M: int, prec: int) -> float:
-    """Algorithmic bytes per pixel and tick: state read + written (8 values
-    per component: 4 bytes each in FP32, 2 in FP16/BF16), RGB (3) + depth (2)
-    read, the List-1 byte read and written (2), one mask bit (1/8)."""
+    """Bytes per pixel and tick when the whole state moves: state read +
+    written (8 values per component: 4 bytes each in FP32, 2 in FP16/BF16), RGB
+    (3) + depth (2) read, the List-1 byte read and written (2), one mask bit
+    (1/8)."""
     per_comp = 64 if prec == 0 else 32
     return per_comp * M + 3 + 2 + 2 + 0.125
+
+
+def needed_bytes_per_pixel(M: int, prec: int) -> float:
+    """Bytes per pixel a tick cannot do without: every weight read and written
+    and every variance read (6 values per component), the mean of one
+    component per mixture read (4) and its mean and variance written (6), and
+    the frame, List-1 byte and mask bit as in bytes_per_pixel. The means and
+    variances of the other components do not change."""
+    return (6 * M + 10) * (4 if prec == 0 else 2) + 3 + 2 + 2 + 0.125
 
 
 def kernel_source_hash(sources=None) -> str:
@@ -509,7 +525,7 @@ def run_gmm(args, wl):
     # a separate pass times a handle without the opening back to back (the
     # tick's duration), then steps of tick + gmm_morph_open3 with events
     # around the opening (its own duration; the events add a little to it).
-    bpp = bytes_per_pixel(M, prec)
+    bpp = needed_bytes_per_pixel(M, prec)
     morph_info = None
     if args.morph:
         n_att = min(K, 2000)
@@ -592,9 +608,10 @@ def run_gmm(args, wl):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
                          "peak_source": peak_src, "algorithmic_bytes_per_px": bpp,
+                         "whole_state_bytes_per_px": bytes_per_pixel(M, prec),
                          "kernel": (f"k_tick_staged<M={M},{'f32' if prec == 0 else 'f16'}>"
                                     f" variant {args.variant}" if args.kernel == "staged" else
-                                    f"k_tick_{'f32' if prec == 0 else 'f16'}<M={M}>")},
+                                    f"k_tick<M={M},{'f32' if prec == 0 else 'f16'}>")},
             "latency_ms": {"tick_p50": pct(tick_sorted, 50), "tick_p99": pct(tick_sorted, 99),
                            "e2e_p50": e2e["lat_p50"], "e2e_p99": e2e["lat_p99"]},
             "e2e": {"value": e2e["value"], "unit": UNIT, "h2d_bytes_per_step": e2e["h2d"],
@@ -634,7 +651,7 @@ def camera_mix(cams_per_res: int, rank: int):
     return out
 
 
-def pool_config(key, wl, world, cams, shape, graph):
+def pool_config(key, wl, world, cams, shape):
     px = sum(H * W for (H, W, _, _) in cams)
     state = sum(H * W * M * (32 if wl["prec"] == 0 else 16) for (H, W, M, _) in cams)
     return {"workload": f"{key}: {wl['name']}", "cameras_per_gpu": len(cams),
@@ -642,7 +659,7 @@ def pool_config(key, wl, world, cams, shape, graph):
             "M5_cameras": sum(1 for c in cams if c[2] == 5),
             "state": "f32" if wl["prec"] == 0 else "f16/bf16",
             "alpha": PARAMS["alpha"], "k": PARAMS["match_k"], "T": PARAMS["bg_T"],
-            "launch": shape, "cuda_graph": graph, "parallelism": f"camera-sharded x{world}",
+            "launch": shape, "parallelism": f"camera-sharded x{world}",
             "l2": f"state {state / 1e9:.1f} GB per GPU vs L2 129 MB: inputs larger than L2 "
                   "between iterations"}
 
@@ -664,8 +681,19 @@ def run_pool(args, wl):
     K, Wm = args.steps, args.warmup
     stream = torch.cuda.current_stream(dev)
     frames = []
+    prm = dict(PARAMS)
+    if args.scene == "strobe":
+        nf = 15  # whole cycles of 3 and of 5 values
+        prm.update(alpha=0.1, init_w=0.5)  # a value outranks the others at once
+        wl = dict(wl, name=wl["name"] + " [strobe: constant frames cycling through M values]")
     for (H, W, M, seed) in cams:
-        r, d, _ = synth.frames_device(synth.scene(seed, H, W, 1), 0, nf, device=dev, with_gt=False)
+        if args.scene == "strobe":
+            v = torch.arange(nf, device=dev) % M
+            r = (20 + 50 * v).to(torch.uint8).view(nf, 1, 1, 1).expand(nf, H, W, 3).contiguous()
+            d = (1000 + 500 * v).to(torch.int16).view(nf, 1, 1).expand(nf, H, W).contiguous()
+        else:
+            r, d, _ = synth.frames_device(synth.scene(seed, H, W, 1), 0, nf, device=dev,
+                                          with_gt=False)
         frames.append((r, d))
     masks = [torch.empty((H, G.mask_words_per_row(W)), dtype=torch.int32, device=dev)
              for (H, W, _, _) in cams]
@@ -677,10 +705,8 @@ def run_pool(args, wl):
     mask_ptr = [m.data_ptr() for m in masks]
 
     pool = G.Pool(precision=prec, max_cams=len(cams), device=dev)
-    ids = [pool.admit(H, W, M, flags=model_flags(args, G), **PARAMS) for (H, W, M, _) in cams]
+    ids = [pool.admit(H, W, M, flags=model_flags(args, G), **prm) for (H, W, M, _) in cams]
     pool.set_stream(stream)
-    graph = not args.no_graph
-    pool.use_graph(graph)
 
     def submit(f):
         pool.submit_many(ids, [b + f * s for b, s in zip(rgb_base, rgb_step)],
@@ -735,15 +761,16 @@ def run_pool(args, wl):
     total_ms = reduce_max(local_ms, world, dev)
     px = sum(H * W for (H, W, _, _) in cams)
     value = aggregate_mpx_per_s(world, K, px, total_ms)
-    tick_bytes = sum(H * W * bytes_per_pixel(M, prec) for (H, W, M, _) in cams)
+    tick_bytes = sum(H * W * needed_bytes_per_pixel(M, prec) for (H, W, M, _) in cams)
     achieved = tick_bytes / (local_ms / K / 1e3) / 1e9
     # one launch per tick up to 128 cameras (more: a launch per 128)
     flat = bool(shape) and shape.get("ctas_per_sm", 0) < 0
-    traffic = recorded_traffic("pool_full", prec, tick_bytes, exact=True) if not flat else None
+    traffic = (recorded_traffic("pool_scene", prec, tick_bytes, exact=True)
+               if not flat and args.scene == "frames" else None)
     traffic_note = "one-pass ncu capture of this 64-camera launch"
     if traffic is None:
         traffic = (recorded_traffic("pool_flat" if flat else "pool", prec, tick_bytes)
-                   if len(cams) <= 128 else None)
+                   if len(cams) <= 128 and args.scene == "frames" else None)
         traffic_note = "scaled from an 8-camera capture by algorithmic bytes"
     peak, peak_src = measured_hbm_peak()
 
@@ -800,7 +827,7 @@ def run_pool(args, wl):
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K,
             "warmup": Wm, "ms_per_step": total_ms / K, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
-            "config": pool_config(args.workload, wl, world, cams, shape, graph),
+            "config": pool_config(args.workload, wl, world, cams, shape),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic, "peak_source": peak_src,
                          "traffic_note": traffic_note,
@@ -815,7 +842,7 @@ def run_pool(args, wl):
                     "d2h_bytes_per_step": e2e["d2h"], "launch": e2e["launch"],
                     "path": "pinned packed tick-sets -> device staging (copy stream) -> "
                             "gmm_pool_submit_many + gmm_pool_tick -> masks to pinned host "
-                            "(FP16/BF16 next-tile prefetch off; the launch shape tuned in "
+                            "(FP16/BF16 prefetch off; the launch shape tuned in "
                             "this pipeline unless fixed)"},
             "e2e_zero_copy": {"value": e2e["zero_copy"], "unit": UNIT,
                               "h2d_bytes_per_step": e2e["h2d"], "d2h_bytes_per_step": e2e["d2h"],
@@ -851,7 +878,6 @@ def pool_precision_extra(G, torch, args, cams, rgb_base, dep_base, rgb_step, dep
     pool = G.Pool(precision=prec, max_cams=len(cams), device=stream.device)
     ids = [pool.admit(H, W, M, **PARAMS) for (H, W, M, _) in cams]
     pool.set_stream(stream)
-    pool.use_graph(True)
 
     def submit(f):
         pool.submit_many(ids, [b + f * s for b, s in zip(rgb_base, rgb_step)],
@@ -881,7 +907,7 @@ def pool_precision_extra(G, torch, args, cams, rgb_base, dep_base, rgb_step, dep
     shape = pool.tuning()[1]
     pool.close()
     px = sum(H * W for (H, W, _, _) in cams)
-    tick_bytes = sum(H * W * bytes_per_pixel(M, prec) for (H, W, M, _) in cams)
+    tick_bytes = sum(H * W * needed_bytes_per_pixel(M, prec) for (H, W, M, _) in cams)
     achieved = tick_bytes / (ms / steps / 1e3) / 1e9
     peak, peak_src = measured_hbm_peak()
     flat = shape.get("ctas_per_sm", 0) < 0
@@ -891,7 +917,7 @@ def pool_precision_extra(G, torch, args, cams, rgb_base, dep_base, rgb_step, dep
             "launch": shape,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "peak_source": peak_src,
-                         "traffic": (recorded_traffic("pool_full", prec, tick_bytes, exact=True)
+                         "traffic": (recorded_traffic("pool_scene", prec, tick_bytes, exact=True)
                                      if not flat else None)
                                     or (recorded_traffic("pool_flat" if flat else "pool", prec,
                                                          tick_bytes) if len(cams) <= 128 else None),
@@ -1349,7 +1375,7 @@ def run_serving(args, wl):
     ev3 = serving_schedule(len(cams), wl["tight_duration_s"], wl["fps"],
                            wl["session_frames"] / wl["fps"], wl["live_fraction"], 2021 + rank, True)
     burst_px = sum(cams[c][0] * cams[c][1] for (t, kind, c, _) in ev3 if t == 0.0 and kind == 0)
-    mean_bpp = sum(H * W * bytes_per_pixel(M, wl["prec"]) for (H, W, M, _) in cams) / \
+    mean_bpp = sum(H * W * needed_bytes_per_pixel(M, wl["prec"]) for (H, W, M, _) in cams) / \
         sum(H * W for (H, W, _, _) in cams)
     achieved = pixels * mean_bpp / wall / 1e9
     peak, peak_src = measured_hbm_peak()
@@ -1503,7 +1529,10 @@ def main(argv=None):
                     help="override the workload's state storage precision")
     ap.add_argument("--cams-per-res", type=int, default=0,
                     help="pooled workloads: cameras per resolution (0: the workload's 16)")
-    ap.add_argument("--no-graph", action="store_true", help="pooled workloads: no CUDA graph")
+    ap.add_argument("--scene", choices=["frames", "strobe"], default="frames",
+                    help="pooled workloads: the workload's synthetic frames, or constant frames "
+                         "cycling through M values per camera, so that every tick matches the "
+                         "last-ranked component and moves the whole state (traffic captures)")
     ap.add_argument("--serve-seconds", type=float, default=0.0,
                     help="serving workload: simulated seconds (0: the workload's 20)")
     ap.add_argument("--serve-copy", action="store_true",
