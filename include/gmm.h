@@ -391,6 +391,8 @@ int gmm_pool_tick(gmm_pool_t *p);
 /* As gmm_inject_cuda_error, for a pool: later ticks return GMM_ECUDA. */
 int gmm_pool_inject_cuda_error(gmm_pool_t *p, int cuda_error);
 
+/* Stream for all later work of the pool. A tick follows the pool's last one
+ * also where that ran on another stream. Ticks cannot be captured (GMM_ECUDA). */
 int gmm_pool_set_stream(gmm_pool_t *p, void *cuda_stream);
 
 /* Launch shape of the pooled kernel: threads per block (64..256, a

@@ -74,6 +74,11 @@ struct gmm_pool {
     int prec = 0, max_cams = 0, device = 0;
     std::vector<PoolCam> cams;
     cudaStream_t stream = nullptr;
+    // Ticks follow one another when the stream changes between them: the stream
+    // of the last tick, and an event behind it.
+    cudaStream_t tick_stream = nullptr;
+    cudaEvent_t ev_tick = nullptr;
+    bool ticked = false;
     cudaMemPool_t mempool = nullptr;   // cameras' state; keeps freed memory mapped
     cudaError_t sticky = cudaSuccess;
     int threads = 128, ctas_per_sm = 0, tile_pixels = 2048; // ctas_per_sm < 0: flat form
@@ -187,17 +192,36 @@ static int tuning_poll(gmm_pool *p, bool block) {
     return GMM_OK;
 }
 
+// A tick reads the state and the tile counters that the tick before it wrote,
+// on whatever stream that was. An event between two ticks costs them their
+// programmatic overlap, so none is recorded on the legacy stream, which always
+// exists and can be recorded later; another stream may be gone by then.
+static cudaError_t order_before_tick(gmm_pool *p) {
+    if (!p->ticked || p->tick_stream == p->stream)
+        return cudaSuccess;
+    cudaError_t e = p->tick_stream ? cudaSuccess : cudaEventRecord(p->ev_tick, nullptr);
+    return e == cudaSuccess ? cudaStreamWaitEvent(p->stream, p->ev_tick, 0) : e;
+}
+
+static cudaError_t order_after_tick(gmm_pool *p) {
+    p->ticked = true;
+    p->tick_stream = p->stream;
+    return p->stream ? cudaEventRecord(p->ev_tick, p->stream) : cudaSuccess;
+}
+
 // Launch the tick's n_launch launches.
 static cudaError_t launch_tick(gmm_pool *p, int n_launch, bool all_variants) {
     const bool flat = p->ctas_per_sm < 0;
     const int warps = p->threads / 32;
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = order_before_tick(p);
     for (int li = 0; li < n_launch && e == cudaSuccess; ++li) {
         const gmmhost::PoolArgs &a = p->args[li];
         const int blocks = flat ? (int)((a.n_tiles + warps - 1) / warps) : blocks_for(p);
         e = gmmhost::launch_pool_tick_impl(a, p->threads, blocks, p->prec, all_variants, flat,
                                            p->launch_m[li], p->prefetch, p->stream);
     }
+    if (e == cudaSuccess)
+        e = order_after_tick(p);
     return e;
 }
 
@@ -356,8 +380,16 @@ gmm_pool_t *gmm_pool_create(size_t budget_bytes, int precision, int max_cams) {
     // one launch per kPoolViews cameras, plus one per M group in the flat form
     p->kmax = (max_cams + gmmhost::kPoolViews - 1) / gmmhost::kPoolViews + 2;
     p->launch_m.assign((size_t)p->kmax, 0);
-    p->args.resize((size_t)p->kmax);
+    try {
+        p->args.resize((size_t)p->kmax);
+    } catch (const std::bad_alloc &) {
+        fail(GMM_ENOMEM, "gmm_pool_create: host allocation failed");
+        delete p;
+        return nullptr;
+    }
     cudaError_t e = cudaGetDevice(&p->device);
+    if (e == cudaSuccess)
+        e = cudaEventCreateWithFlags(&p->ev_tick, cudaEventDisableTiming);
     if (e == cudaSuccess)
         e = cudaMalloc(&p->d_counters, sizeof(int) * 2 * (size_t)p->kmax);
     if (e == cudaSuccess)
@@ -495,6 +527,14 @@ int gmm_pool_tick(gmm_pool_t *p) {
         return fail(GMM_ECUDA, std::string("gmm_pool_tick: earlier CUDA failure: ") +
                                    cudaGetErrorString(p->sticky));
     DeviceGuard g(p->device);
+    // A captured tick would replay with this tick's tile counters, which are
+    // zero only once.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(p->stream, &cap);
+    if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return fail(GMM_ECUDA, "gmm_pool_tick: a pool's ticks cannot be captured");
+    }
     return pool_tick_impl(p, true);
 }
 
@@ -736,6 +776,8 @@ int gmm_pool_destroy(gmm_pool_t *p) {
         cudaMemPoolDestroy(p->mempool);
     if (p->d_counters)
         cudaFree(p->d_counters);
+    if (p->ev_tick)
+        cudaEventDestroy(p->ev_tick);
     delete p;
     return GMM_OK;
 }
