@@ -637,8 +637,9 @@ int gmm_pipe_wait(gmm_t *h, long long ticket, int timeout_ms) {
 }
 
 // Whether the tick may read the frame from, and write the mask to, these host
-// buffers in place: page-locked memory mapped at the same address, aligned as
-// the kernels need it, the mask apart from the frame.
+// buffers in place: page-locked memory mapped at the same address, from the
+// first byte to the last, aligned as the kernels need it, the mask apart from
+// the frame.
 static bool in_place(const gmm_ctx *h, const uint8_t *rgb, const uint16_t *depth,
                      const uint32_t *mask) {
     const size_t N = (size_t)h->cfg.H * h->cfg.W;
@@ -647,8 +648,8 @@ static bool in_place(const gmm_ctx *h, const uint8_t *rgb, const uint16_t *depth
                     m1 = m + (size_t)h->cfg.H * h->L.wpr * 4;
     if (d % 2 || m % 4 || (r < m1 && m < r + 3 * N) || (d < m1 && m < d + 2 * N))
         return false;
-    for (const void *p : {static_cast<const void *>(rgb), static_cast<const void *>(depth),
-                          static_cast<const void *>(mask)}) {
+    for (const uintptr_t q : {r, r + 3 * N - 1, d, d + 2 * N - 1, m, m1 - 1}) {
+        void *p = reinterpret_cast<void *>(q);
         cudaPointerAttributes a;
         if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
             cudaGetLastError();
