@@ -212,6 +212,8 @@ def _stream_ptr(stream, device) -> int:
     global _raw_stream
     if stream is not None:
         return stream.cuda_stream
+    if device.type != "cuda":
+        raise ValueError(f"expected a CUDA device, got {device}")
     if _raw_stream is None:
         import torch
         _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (

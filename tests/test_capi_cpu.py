@@ -172,3 +172,11 @@ def test_server_stats_struct_matches_header():
         names += [n.strip() for n in decl.split(",")]
     assert names == [f[0] for f in G.ServerStats._fields_]
     assert ctypes.sizeof(G.ServerStats) == 8 * 8 + 8 + 8 * 2 + 8
+
+
+def test_current_stream_of_a_cpu_device_is_refused():
+    import torch
+    with pytest.raises(ValueError):
+        G._stream_ptr(None, torch.device("cpu"))
+    with pytest.raises(ValueError):
+        G._stream_ptr(None, torch.device("cpu", 0))
