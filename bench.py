@@ -431,7 +431,7 @@ def run_reference(args, wl):
     value, dt = oracle_parallel(bands, args.warmup, args.steps, procs)
     sample = ("each step: " + "; ".join(descr) + f" (one frame each), FP64, {procs} processes "
               "over row bands")
-    cfg = (pool_config(args.workload, wl, world, camera_mix(wl["cams_per_res"], 0), None, None)
+    cfg = (pool_config(args.workload, wl, world, camera_mix(wl["cams_per_res"], 0), None)
            if (wl.get("pool") or wl.get("serve")) else config_dict(args.workload, wl, world))
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "impl": "reference", "n_gpus": world,
