@@ -391,8 +391,12 @@ int gmm_pool_tick(gmm_pool_t *p);
 /* As gmm_inject_cuda_error, for a pool: later ticks return GMM_ECUDA. */
 int gmm_pool_inject_cuda_error(gmm_pool_t *p, int cuda_error);
 
-/* Stream for all later work of the pool. A tick follows the pool's last one
- * also where that ran on another stream. Ticks cannot be captured (GMM_ECUDA). */
+/* Stream for all later work of the pool. Work on the pool (ticks, admissions,
+ * releases, state reads) follows the pool's work before it also where that ran
+ * on another stream, whatever the handles (cudaStreamPerThread of another
+ * thread, a stream since destroyed); a thread whose cudaStreamPerThread was
+ * used stays until the work on it is done. Ticks cannot be captured
+ * (GMM_ECUDA). */
 int gmm_pool_set_stream(gmm_pool_t *p, void *cuda_stream);
 
 /* Launch shape of the pooled kernel: threads per block (64..256, a
@@ -466,7 +470,7 @@ size_t gmm_pool_state_used(const gmm_pool_t *p);
  * supply it, GMM_ECUDA on another CUDA failure (not sticky). */
 int gmm_pool_reserve(gmm_pool_t *p, size_t bytes);
 
-/* Wait for every tick queued on the pool's stream. GMM_ECUDA if a CUDA
+/* Wait for the pool's stream and for every tick queued. GMM_ECUDA if a CUDA
  * failure is sticky on the pool. */
 int gmm_pool_sync(gmm_pool_t *p);
 

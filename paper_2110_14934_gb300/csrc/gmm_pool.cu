@@ -74,11 +74,10 @@ struct gmm_pool {
     int prec = 0, max_cams = 0, device = 0;
     std::vector<PoolCam> cams;
     cudaStream_t stream = nullptr;
-    // Ticks follow one another when the stream changes between them: the stream
-    // of the last tick, and an event behind it.
-    cudaStream_t tick_stream = nullptr;
-    cudaEvent_t ev_tick = nullptr;
-    bool ticked = false;
+    // The last work on the pool's state: whether there is any, whether it went
+    // to the legacy stream, and else an event behind it (order_before).
+    bool worked = false, worked_on_legacy = false;
+    cudaEvent_t ev_work = nullptr;
     cudaMemPool_t mempool = nullptr;   // cameras' state; keeps freed memory mapped
     cudaError_t sticky = cudaSuccess;
     int threads = 128, ctas_per_sm = 0, tile_pixels = 2048; // ctas_per_sm < 0: flat form
@@ -192,28 +191,42 @@ static int tuning_poll(gmm_pool *p, bool block) {
     return GMM_OK;
 }
 
-// A tick reads the state and the tile counters that the tick before it wrote,
-// on whatever stream that was. An event between two ticks costs them their
-// programmatic overlap, so none is recorded on the legacy stream, which always
-// exists and can be recorded later; another stream may be gone by then.
-static cudaError_t order_before_tick(gmm_pool *p) {
-    if (!p->ticked || p->tick_stream == p->stream)
+// Work on a pool's state and tile counters (ticks, admissions, releases, state
+// reads) follows the pool's work before it, on whatever stream that was. The
+// handles do not say whether it was the same one: cudaStreamPerThread is
+// another stream in every thread, and a destroyed stream's handle may come back
+// for a new one while the old one's work is still queued. So work on any stream
+// but the legacy one leaves an event behind it, and the next work waits for it
+// (ticks on one created stream, with and without that wait: 12 cameras of
+// 320x240 20.2-20.4 and 20.4-20.6 us, 24 FP16/BF16 cameras of odd sizes 275 and
+// 275; the event alone parts them). The legacy stream is one per device and always
+// exists: work that stays on it needs no event, which would cost consecutive
+// ticks their programmatic overlap, and it can be recorded later.
+static cudaError_t order_before(gmm_pool *p) {
+    if (!p->worked || (p->worked_on_legacy && !p->stream))
         return cudaSuccess;
-    cudaError_t e = p->tick_stream ? cudaSuccess : cudaEventRecord(p->ev_tick, nullptr);
-    return e == cudaSuccess ? cudaStreamWaitEvent(p->stream, p->ev_tick, 0) : e;
+    cudaError_t e = p->worked_on_legacy ? cudaEventRecord(p->ev_work, nullptr) : cudaSuccess;
+    return e == cudaSuccess ? cudaStreamWaitEvent(p->stream, p->ev_work, 0) : e;
 }
 
-static cudaError_t order_after_tick(gmm_pool *p) {
-    p->ticked = true;
-    p->tick_stream = p->stream;
-    return p->stream ? cudaEventRecord(p->ev_tick, p->stream) : cudaSuccess;
+static cudaError_t order_after(gmm_pool *p) {
+    p->worked = true;
+    p->worked_on_legacy = !p->stream;
+    return p->stream ? cudaEventRecord(p->ev_work, p->stream) : cudaSuccess;
+}
+
+// The host waits for the pool's last work, without using its stream.
+static cudaError_t wait_for_work(const gmm_pool *p) {
+    if (!p->worked)
+        return cudaSuccess;
+    return p->worked_on_legacy ? cudaStreamSynchronize(nullptr) : cudaEventSynchronize(p->ev_work);
 }
 
 // Launch the tick's n_launch launches.
 static cudaError_t launch_tick(gmm_pool *p, int n_launch, bool all_variants) {
     const bool flat = p->ctas_per_sm < 0;
     const int warps = p->threads / 32;
-    cudaError_t e = order_before_tick(p);
+    cudaError_t e = order_before(p);
     for (int li = 0; li < n_launch && e == cudaSuccess; ++li) {
         const gmmhost::PoolArgs &a = p->args[li];
         const int blocks = flat ? (int)((a.n_tiles + warps - 1) / warps) : blocks_for(p);
@@ -221,7 +234,7 @@ static cudaError_t launch_tick(gmm_pool *p, int n_launch, bool all_variants) {
                                            p->launch_m[li], p->prefetch, p->stream);
     }
     if (e == cudaSuccess)
-        e = order_after_tick(p);
+        e = order_after(p);
     return e;
 }
 
@@ -389,7 +402,7 @@ gmm_pool_t *gmm_pool_create(size_t budget_bytes, int precision, int max_cams) {
     }
     cudaError_t e = cudaGetDevice(&p->device);
     if (e == cudaSuccess)
-        e = cudaEventCreateWithFlags(&p->ev_tick, cudaEventDisableTiming);
+        e = cudaEventCreateWithFlags(&p->ev_work, cudaEventDisableTiming);
     if (e == cudaSuccess)
         e = cudaMalloc(&p->d_counters, sizeof(int) * 2 * (size_t)p->kmax);
     if (e == cudaSuccess)
@@ -430,9 +443,13 @@ int gmm_pool_admit(gmm_pool_t *p, const gmm_config *cfg) {
         return fail(GMM_ENOMEM, "gmm_pool_admit: every slot is taken");
     DeviceGuard g(p->device);
     void *arena = nullptr;
-    cudaError_t e = cudaMallocFromPoolAsync(&arena, L.total, p->mempool, p->stream);
+    cudaError_t e = order_before(p);
+    if (e == cudaSuccess)
+        e = cudaMallocFromPoolAsync(&arena, L.total, p->mempool, p->stream);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(arena, 0, L.total, p->stream);
+    if (e == cudaSuccess)
+        e = order_after(p);
     if (e != cudaSuccess) {
         cudaGetLastError();
         if (arena)
@@ -471,7 +488,11 @@ int gmm_pool_release(gmm_pool_t *p, int cam) {
     DeviceGuard g(p->device);
     PoolCam &c = p->cams[cam];
     // Stream-ordered free: queued ticks that use the state run first.
-    const cudaError_t e = cudaFreeAsync(c.arena, p->stream);
+    cudaError_t e = order_before(p);
+    if (e == cudaSuccess)
+        e = cudaFreeAsync(c.arena, p->stream);
+    if (e == cudaSuccess)
+        e = order_after(p);
     p->used_bytes -= c.L.total;
     c = PoolCam();
     if (e != cudaSuccess)
@@ -644,6 +665,7 @@ int gmm_pool_autotune(gmm_pool_t *p, int iters, int *threads_out, int *ctas_out,
     }
     std::vector<int> init_saved(p->cams.size());
     size_t off = 0;
+    e = order_before(p);
     for (size_t i = 0; i < p->cams.size() && e == cudaSuccess; ++i) {
         PoolCam &c = p->cams[i];
         init_saved[i] = c.initialized;
@@ -739,6 +761,9 @@ int gmm_pool_state_get(const gmm_pool_t *p, int cam, int plane, int component,
     DeviceGuard g(p->device);
     gmm_pool *pm = const_cast<gmm_pool *>(p);
     const PoolCam &c = p->cams[cam];
+    const cudaError_t e = order_before(pm);
+    if (e != cudaSuccess)
+        return cuda_fail(&pm->sticky, e, "gmm_pool_state_get");
     return state_get_common(c.cfg, c.L, c.arena, p->stream, &pm->sticky, plane, component,
                             dst_host, n);
 }
@@ -749,7 +774,9 @@ int gmm_pool_sync(gmm_pool_t *p) {
     if (!p)
         return fail(GMM_EINVAL, "gmm_pool_sync: null pool");
     DeviceGuard g(p->device);
-    const cudaError_t e = cudaStreamSynchronize(p->stream);
+    cudaError_t e = cudaStreamSynchronize(p->stream);
+    if (e == cudaSuccess)
+        e = wait_for_work(p); // it may have gone to an earlier stream
     if (e != cudaSuccess)
         return cuda_fail(&p->sticky, e, "gmm_pool_sync");
     return p->sticky == cudaSuccess ? GMM_OK : fail(GMM_ECUDA, "gmm_pool_sync: earlier CUDA failure");
@@ -760,6 +787,7 @@ int gmm_pool_destroy(gmm_pool_t *p) {
         return fail(GMM_EINVAL, "gmm_pool_destroy: null pool");
     DeviceGuard g(p->device);
     cudaStreamSynchronize(p->stream);
+    wait_for_work(p);
     for (Trial &tr : p->tune.pending) {
         cudaEventDestroy(tr.a);
         cudaEventDestroy(tr.b);
@@ -776,8 +804,8 @@ int gmm_pool_destroy(gmm_pool_t *p) {
         cudaMemPoolDestroy(p->mempool);
     if (p->d_counters)
         cudaFree(p->d_counters);
-    if (p->ev_tick)
-        cudaEventDestroy(p->ev_tick);
+    if (p->ev_work)
+        cudaEventDestroy(p->ev_work);
     delete p;
     return GMM_OK;
 }
