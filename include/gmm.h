@@ -223,10 +223,11 @@ int gmm_apply_ex(gmm_t *h, const uint8_t *rgb8, const uint16_t *depth16,
  * tick). rgb8_host, depth16_host: host, read; mask_host: host, written.
  * Copies the frame in, runs gmm_apply, copies the mask out, and returns when
  * the mask is in host memory. Staging buffers are owned by the handle and
- * allocated on first use. With page-locked buffers mapped into the device's
- * address space (depth16_host 2-byte and mask_host 4-byte aligned, the mask
- * apart from the frame) and no gmm_pipe_submit frame in flight, the tick reads
- * the frame and writes the mask in place instead, without copies. */
+ * allocated on first use. With buffers that are page-locked and mapped into
+ * the device's address space to their last byte (depth16_host 2-byte and
+ * mask_host 4-byte aligned, the mask apart from the frame), the direct kernel
+ * and no gmm_pipe_submit frame in flight, the tick reads the frame and writes
+ * the mask in place instead, without copies. */
 int gmm_apply_host(gmm_t *h, const uint8_t *rgb8_host,
                    const uint16_t *depth16_host, uint32_t *mask_host);
 

@@ -1,5 +1,6 @@
 // C ABI of the single-camera model: argument checks, device state ownership,
 // launches, state transfer and the pipelined host-memory path.
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -14,6 +15,7 @@
 
 #include "gmm.h"
 #include "gmm_common.h"
+#include "gmm_host_frames.h"
 #include "gmm_internal.h"
 
 using gmmdev::CamView;
@@ -636,29 +638,43 @@ int gmm_pipe_wait(gmm_t *h, long long ticket, int timeout_ms) {
     return rc;
 }
 
-// Whether the tick may read the frame from, and write the mask to, these host
-// buffers in place: page-locked memory mapped at the same address, from the
-// first byte to the last, aligned as the kernels need it, the mask apart from
-// the frame.
+// The page-locked span that holds q, mapped at the same addresses (one driver
+// query; through the entry point the runtime hands out, no link against
+// libcuda).
+static HostSpan page_locked_span(uintptr_t q) {
+    static const auto query = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn,
+                                                               12000, cudaEnableDefault, &r);
+        if (e != cudaSuccess || r != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<decltype(&cuPointerGetAttributes)>(fn);
+    }();
+    unsigned type = 0, managed = 0;
+    CUdeviceptr dev = 0, base = 0;
+    size_t size = 0;
+    CUpointer_attribute attrs[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE,
+                                   CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                   CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                   CU_POINTER_ATTRIBUTE_MAPPING_BASE_ADDR,
+                                   CU_POINTER_ATTRIBUTE_MAPPING_SIZE};
+    void *out[] = {&type, &managed, &dev, &base, &size};
+    if (!query || query(5, attrs, out, (CUdeviceptr)q) != CUDA_SUCCESS ||
+        type != CU_MEMORYTYPE_HOST || managed || dev != (CUdeviceptr)q)
+        return {q, q};
+    return {(uintptr_t)base, (uintptr_t)base + size};
+}
+
+// (frame_in_place says which frames qualify.)
 static bool in_place(const gmm_ctx *h, const uint8_t *rgb, const uint16_t *depth,
                      const uint32_t *mask) {
-    const size_t N = (size_t)h->cfg.H * h->cfg.W;
-    const uintptr_t r = reinterpret_cast<uintptr_t>(rgb), d = reinterpret_cast<uintptr_t>(depth),
-                    m = reinterpret_cast<uintptr_t>(mask),
-                    m1 = m + (size_t)h->cfg.H * h->L.wpr * 4;
-    if (d % 2 || m % 4 || (r < m1 && m < r + 3 * N) || (d < m1 && m < d + 2 * N))
-        return false;
-    for (const uintptr_t q : {r, r + 3 * N - 1, d, d + 2 * N - 1, m, m1 - 1}) {
-        void *p = reinterpret_cast<void *>(q);
-        cudaPointerAttributes a;
-        if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        if (a.type != cudaMemoryTypeHost || a.devicePointer != p)
-            return false;
-    }
-    return true;
+    return frame_in_place(h->kernel == GMM_KERNEL_STAGED, reinterpret_cast<uintptr_t>(rgb),
+                          reinterpret_cast<uintptr_t>(depth), reinterpret_cast<uintptr_t>(mask),
+                          (size_t)h->cfg.H * h->cfg.W, (size_t)h->cfg.H * h->L.wpr * 4,
+                          page_locked_span);
 }
 
 // With page-locked buffers and no queued frame in flight, the tick works on
