@@ -403,10 +403,10 @@ int gmm_pool_set_stream(gmm_pool_t *p, void *cuda_stream);
 /* Launch shape of the pooled kernel: threads per block (64..256, a
  * multiple of 32); CTAs per SM of the persistent form (>= 1; its CTAs loop
  * over tiles of tile_pixels pixels, a multiple of the block size, or of
- * fewer where a tick has too few pixels for such tiles to occupy every CTA
- * evenly), or -1 for the flat form (a grid over the launch's pixels in which every warp
- * takes one chunk of 32 pixels, FP32, or 64, FP16/BF16, and exits;
- * tile_pixels is then unused). 0 keeps the current value (initially: 128
+ * fewer where a launch has too few pixels for such tiles to occupy every
+ * CTA evenly), or -1 for the flat form (a grid over the launch's pixels in
+ * which every warp takes one chunk of 32 pixels, FP32, or 64, FP16/BF16, and
+ * exits; tile_pixels is then unused). 0 keeps the current value (initially: 128
  * threads, as many persistent CTAs as fit, 2048-pixel tiles). */
 int gmm_pool_set_launch(gmm_pool_t *p, int threads, int ctas_per_sm,
                         int tile_pixels);
@@ -432,8 +432,10 @@ int gmm_pool_autotune(gmm_pool_t *p, int iters, int *threads,
 /* Online tuning of the launch shape on real ticks: the next
  * ticks_per_shape x (number of candidates) calls of gmm_pool_tick each run
  * one candidate shape (block size 64/128/256; the persistent form at full or
- * half residency with tiles of 256/512/1024/2048/8192 pixels; round-robin;
- * the flat form is chosen only explicitly). Each such tick is timed on the
+ * half residency with tiles of 256/512/1024/2048/8192 pixels, or fewer shapes
+ * where the first of these ticks runs smaller tiles than that: each that runs
+ * once, under the tile size it runs with; round-robin; the flat form is
+ * chosen only explicitly). Each such tick is timed on the
  * pool's stream from its start to the start of the next tick (the tick
  * period, so whatever the tick's kernel delays among the work queued before
  * the next tick, such as uploads of the next frames, counts against its

@@ -13,6 +13,7 @@
 #include "gmm.h"
 #include "gmm_common.h"
 #include "gmm_internal.h"
+#include "gmm_pool_plan.h"
 
 using gmmdev::CamView;
 using namespace gmmlib;
@@ -32,10 +33,7 @@ struct PoolCam {
     uint32_t *mask = nullptr, *fgr = nullptr, *fgd = nullptr;
 };
 
-// ctas < 0: the flat (non-persistent) form; tile is then its chunk size.
-struct Shape {
-    int threads, ctas, tile;
-};
+static_assert(kLaunchCams == gmmhost::kPoolViews, "a launch's cameras fit its parameters");
 
 int chunk_pixels(int prec) { return prec == 0 ? 32 : 64; }
 
@@ -56,6 +54,7 @@ constexpr int kFinalists = 4;
 struct Tuning {
     bool active = false;
     bool final_round = false;
+    bool named = false; // cands are the shapes that run (set by the first trial tick)
     int per_shape = 0, issued = 0;
     std::vector<Shape> cands;
     Trial open;                 // the last trial tick, until the next tick starts
@@ -85,23 +84,24 @@ struct gmm_pool {
     // uses set `parity` and its launches zero the other set for the next.
     int *d_counters = nullptr;
     int kmax = 1, parity = 0; // kmax: launches a tick may take
-    std::vector<int> launch_m; // per launch: the M its cameras share (flat form), else 0
-    std::vector<gmmhost::PoolArgs> args; // of a tick's launches (kmax)
+    std::vector<TickCam> tick_cams;      // the tick's cameras, in order of M
+    std::vector<LaunchPlan> plan;        // its launches (at most kmax)
+    std::vector<gmmhost::PoolArgs> args; // and their arguments
     bool prefetch = true; // FP16/BF16: L2 prefetch in the persistent form
     Tuning tune;
     int occupancy[9] = {};  // resident pool CTAs per SM, by block size / 32
     int sms = 0;
 };
 
-// Resident CTAs per SM of the pool kernel for a block size (queried once per
-// block size) times the SM count (queried once).
-static int blocks_for(gmm_pool *p) {
-    int &max_per_sm = p->occupancy[p->threads / 32];
+// CTAs of the persistent form: resident CTAs per SM of the pool kernel for a
+// block size (queried once per block size) times the SM count (queried once).
+static int blocks_for(gmm_pool *p, int threads, int ctas_per_sm) {
+    int &max_per_sm = p->occupancy[threads / 32];
     if (max_per_sm == 0)
-        max_per_sm = gmmhost::pool_max_ctas_per_sm(p->prec, p->threads);
+        max_per_sm = gmmhost::pool_max_ctas_per_sm(p->prec, threads);
     if (p->sms == 0)
         p->sms = gmmhost::num_sms();
-    int per_sm = p->ctas_per_sm;
+    int per_sm = ctas_per_sm;
     if (per_sm <= 0 || per_sm > max_per_sm)
         per_sm = max_per_sm;
     if (per_sm < 1)
@@ -109,12 +109,28 @@ static int blocks_for(gmm_pool *p) {
     return p->sms * per_sm;
 }
 
+// The cameras with a submitted frame, in order of M: the flat form launches per
+// M; in the persistent form the CTAs that run together then run one M's body of
+// code (with the cameras mixed, the bodies of all three evict each other from
+// the instruction caches), and the longest tiles come first.
+static const std::vector<TickCam> &submitted_cams(gmm_pool *p) {
+    p->tick_cams.clear();
+    for (int m : {5, 4, 3})
+        for (size_t i = 0; i < p->cams.size(); ++i) {
+            const PoolCam &c = p->cams[i];
+            if (c.used && c.submitted && c.cfg.M == m)
+                p->tick_cams.push_back({(int)i, m, c.L.n_pad});
+        }
+    return p->tick_cams;
+}
+
 // Candidate launch shapes: block sizes, full or half residency, tile sizes
 // of the persistent form. (The flat form is left to an explicit choice: it
 // is the faster one for FP32 state with every input already in device
 // memory, but host uploads that run beside it slow it far more than they
 // slow the persistent form, and ticks timed without such uploads cannot
-// tell.)
+// tell.) A small tick runs smaller tiles than the larger of these
+// (launch_tile): distinct_shapes leaves those that differ on the tick at hand.
 static std::vector<Shape> tuning_candidates(const gmm_pool *p) {
     std::vector<Shape> out;
     const int cand_threads[] = {64, 128, 256};
@@ -222,53 +238,39 @@ static cudaError_t wait_for_work(const gmm_pool *p) {
     return p->worked_on_legacy ? cudaStreamSynchronize(nullptr) : cudaEventSynchronize(p->ev_work);
 }
 
-// Launch the tick's n_launch launches.
-static cudaError_t launch_tick(gmm_pool *p, int n_launch, bool all_variants) {
+// Launch the planned launches.
+static cudaError_t launch_tick(gmm_pool *p, bool all_variants) {
     const bool flat = p->ctas_per_sm < 0;
     const int warps = p->threads / 32;
     cudaError_t e = order_before(p);
-    for (int li = 0; li < n_launch && e == cudaSuccess; ++li) {
+    for (size_t li = 0; li < p->plan.size() && e == cudaSuccess; ++li) {
         const gmmhost::PoolArgs &a = p->args[li];
-        const int blocks = flat ? (int)((a.n_tiles + warps - 1) / warps) : blocks_for(p);
+        const int blocks = flat ? (int)((a.n_tiles + warps - 1) / warps)
+                                : blocks_for(p, p->threads, p->ctas_per_sm);
         e = gmmhost::launch_pool_tick_impl(a, p->threads, blocks, p->prec, all_variants, flat,
-                                           p->launch_m[li], p->prefetch, p->stream);
+                                           p->plan[li].m, p->prefetch, p->stream);
     }
     if (e == cudaSuccess)
         e = order_after(p);
     return e;
 }
 
-// Tile size of a tick of the persistent form: the pool's, or less where that
-// would leave too few tiles or an uneven last wave. share: a CTA's share of the
-// tick's pixels. Large ticks: a sixteenth of it, so the CTAs end together.
-// Smaller ones: about four pixels per thread, in as many equal parts as the
-// share holds. A multiple of the block size. (us per tick, tiles of 256, 512,
-// 896, 2048 pixels: 40 cameras of odd sizes, 29 M pixels, FP16/BF16 477, 442,
-// 429, 427, and 1280 426; 24 cameras, 17 M pixels, FP16/BF16 332, 311, 304, 308,
-// FP32 452, 434, 435, 449; 9 cameras, 6.8 M pixels, FP16/BF16 134, 126, 125,
-// 128; 4 cameras, 3.4 M pixels, FP32 102, 103, 107, 119.)
-static int tick_tile(const gmm_pool *p, int64_t pixels, int blocks) {
-    const int64_t threads = p->threads, four = 4 * threads;
-    const int64_t share = (pixels + blocks - 1) / blocks;
-    int64_t tile = share / 16 / threads * threads;
-    if (tile < four) {
-        const int64_t parts = (share + four - 1) / four;
-        tile = ((share + parts - 1) / parts + threads - 1) / threads * threads;
-    }
-    return tile < p->tile_pixels ? (int)tile : p->tile_pixels;
-}
-
 // One tick over the submitted cameras. clear: drop the submissions and mark
 // the cameras initialised afterwards (false while autotuning).
 static int pool_tick_impl(gmm_pool *p, bool clear) {
-    int64_t pixels = 0;
-    for (const PoolCam &c : p->cams)
-        pixels += (c.used && c.submitted) ? c.L.n_pad : 0;
-    if (pixels == 0)
+    const std::vector<TickCam> &cams = submitted_cams(p);
+    if (cams.empty())
         return GMM_OK;
-    // An online-tuning trial sets its launch shape first: the tile tables
-    // below depend on the tile size.
+    // An online-tuning trial sets its launch shape first: the launches and
+    // their tiles depend on it.
     Tuning &tu = p->tune;
+    if (clear && tu.active && !tu.named) {
+        tu.cands = distinct_shapes(tu.cands, cams, [&](const Shape &s) {
+            return blocks_for(p, s.threads, s.ctas);
+        });
+        tu.ms.assign(tu.cands.size(), {});
+        tu.named = true;
+    }
     const bool trial = clear && tu.active && tu.issued < (int)tu.cands.size() * tu.per_shape;
     Trial tr{};
     if (trial) {
@@ -278,56 +280,34 @@ static int pool_tick_impl(gmm_pool *p, bool clear) {
         p->ctas_per_sm = tu.cands[tr.cand].ctas;
         p->tile_pixels = tu.cands[tr.cand].tile;
     }
-    // The launches' arguments: up to kPoolViews cameras each.
-    // tiles, or in the flat form one chunk per warp
-    const int unit = p->ctas_per_sm < 0 ? chunk_pixels(p->prec)
-                                        : tick_tile(p, pixels, blocks_for(p));
+    // The launches' arguments; tiles, or in the flat form one chunk per warp.
+    const bool flat = p->ctas_per_sm < 0;
+    const Shape shape = {p->threads, p->ctas_per_sm,
+                         flat ? chunk_pixels(p->prec) : p->tile_pixels};
+    plan_launches(cams, shape, flat ? 0 : blocks_for(p, p->threads, p->ctas_per_sm), p->plan);
     int *cur = p->d_counters + p->parity * p->kmax;
     int *next = p->d_counters + (1 - p->parity) * p->kmax;
-    int li = 0, j = 0;
-    int64_t tiles = 0;
     bool all_variants = false; // some camera needs the options or the augmented mixture
-    const bool flat = p->ctas_per_sm < 0;
-    int group_m = 0; // flat form: the launch's cameras share M (a kernel per M)
-    auto close_launch = [&]() {
+    for (size_t li = 0; li < p->plan.size(); ++li) {
+        const LaunchPlan &l = p->plan[li];
         gmmhost::PoolArgs &a = p->args[li];
-        p->launch_m[li] = group_m;
-        a.tile_begin[j] = tiles;
-        a.n_jobs = j;
-        a.n_tiles = tiles;
-        a.tile_pixels = unit;
-        a.counter = cur + li;
-        a.reset = next;
-        a.n_reset = p->kmax;
-        ++li;
-        j = 0;
-        tiles = 0;
-    };
-    // Cameras in order of M: the flat form launches per M; in the persistent
-    // form the CTAs that run together then run one M's body of code (with the
-    // cameras mixed, the bodies of all three evict each other from the
-    // instruction caches), and the longest tiles come first.
-    const int groups[3] = {5, 4, 3};
-    for (int m : groups) {
-        group_m = flat ? m : 0;
-        for (PoolCam &c : p->cams) {
-            if (!(c.used && c.submitted) || c.cfg.M != m)
-                continue;
-            gmmhost::PoolArgs &a = p->args[li];
+        int64_t tiles = 0;
+        for (int j = 0; j < l.count; ++j) {
+            const PoolCam &c = p->cams[cams[l.first + j].slot];
             a.views[j] = make_view(c.cfg, c.L, c.arena, c.rgb, c.depth, c.mask, c.fgr, c.fgd,
                                    c.initialized ? 0 : 1, c.ticks);
             all_variants = all_variants || gmmhost::view_variant(a.views[j]) != 0;
             a.tile_begin[j] = tiles;
-            tiles += (c.L.n_pad + unit - 1) / unit;
-            if (++j == gmmhost::kPoolViews)
-                close_launch();
+            tiles += (c.L.n_pad + l.unit - 1) / l.unit;
         }
-        if (flat && j > 0)
-            close_launch();
+        a.tile_begin[l.count] = tiles;
+        a.n_jobs = l.count;
+        a.n_tiles = tiles;
+        a.tile_pixels = l.unit;
+        a.counter = cur + li;
+        a.reset = next;
+        a.n_reset = p->kmax;
     }
-    if (j > 0)
-        close_launch();
-    const int n_launch = li;
     cudaError_t e = cudaSuccess;
     if (clear && tu.active && tu.open.a) { // this tick's start ends the last trial's period
         e = cudaEventCreate(&tu.open.b);
@@ -350,7 +330,7 @@ static int pool_tick_impl(gmm_pool *p, bool clear) {
         tu.open = tr;
         ++tu.issued;
     }
-    e = launch_tick(p, n_launch, all_variants);
+    e = launch_tick(p, all_variants);
     if (e != cudaSuccess)
         return cuda_fail(&p->sticky, e, "gmm_pool_tick");
     p->parity ^= 1;
@@ -389,11 +369,12 @@ gmm_pool_t *gmm_pool_create(size_t budget_bytes, int precision, int max_cams) {
     p->budget = budget_bytes;
     p->prec = precision;
     p->max_cams = max_cams;
-    p->cams.resize((size_t)max_cams);
-    // one launch per kPoolViews cameras, plus one per M group in the flat form
-    p->kmax = (max_cams + gmmhost::kPoolViews - 1) / gmmhost::kPoolViews + 2;
-    p->launch_m.assign((size_t)p->kmax, 0);
+    // one launch per kLaunchCams cameras, plus one per M group in the flat form
+    p->kmax = (max_cams + kLaunchCams - 1) / kLaunchCams + 2;
     try {
+        p->cams.resize((size_t)max_cams);
+        p->tick_cams.reserve((size_t)max_cams);
+        p->plan.reserve((size_t)p->kmax);
         p->args.resize((size_t)p->kmax);
     } catch (const std::bad_alloc &) {
         fail(GMM_ENOMEM, "gmm_pool_create: host allocation failed");
@@ -618,6 +599,7 @@ int gmm_pool_autotune_online(gmm_pool_t *p, int ticks_per_shape) {
     tu.per_shape = ticks_per_shape;
     tu.issued = 0;
     tu.final_round = false;
+    tu.named = false;
     tu.active = true;
     return GMM_OK;
 }
@@ -682,7 +664,9 @@ int gmm_pool_autotune(gmm_pool_t *p, int iters, int *threads_out, int *ctas_out,
     const int saved_t = p->threads, saved_c = p->ctas_per_sm, saved_tp = p->tile_pixels;
     int best_t = saved_t, best_c = saved_c, best_tp = saved_tp;
     float best_ms = -1.f;
-    const std::vector<Shape> cands = tuning_candidates(p);
+    const std::vector<Shape> cands =
+        distinct_shapes(tuning_candidates(p), submitted_cams(p),
+                        [&](const Shape &s) { return blocks_for(p, s.threads, s.ctas); });
     int rc = GMM_OK;
     // Two passes over the candidates (the best time of each counts), so a
     // transient slowdown during one trial does not decide the shape.
