@@ -259,8 +259,6 @@ static cudaError_t launch_tick(gmm_pool *p, bool all_variants) {
 // the cameras initialised afterwards (false while autotuning).
 static int pool_tick_impl(gmm_pool *p, bool clear) {
     const std::vector<TickCam> &cams = submitted_cams(p);
-    if (cams.empty())
-        return GMM_OK;
     // An online-tuning trial sets its launch shape first: the launches and
     // their tiles depend on it.
     Tuning &tu = p->tune;
@@ -529,6 +527,8 @@ int gmm_pool_tick(gmm_pool_t *p) {
         return fail(GMM_ECUDA, std::string("gmm_pool_tick: earlier CUDA failure: ") +
                                    cudaGetErrorString(p->sticky));
     DeviceGuard g(p->device);
+    if (submitted_cams(p).empty())
+        return GMM_OK; // nothing to launch, on a capturing stream too
     // A captured tick would replay with this tick's tile counters, which are
     // zero only once.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
