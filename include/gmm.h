@@ -513,7 +513,8 @@ typedef struct gmm_server_stats {
     int live_cams;
     size_t budget_bytes, used_bytes;      /* state (+ staging, copy mode) of admitted cameras */
     double max_engine_gap_ms;             /* longest time between two passes of the
-                                             engine's loop (a pass waits at most
+                                             engine's loop, its wait for a queued
+                                             tick's end left out (a pass waits at most
                                              0.2 ms for work; a longer gap means the
                                              thread was blocked, in a CUDA call or a
                                              lock, or not scheduled) */
