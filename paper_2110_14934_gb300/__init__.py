@@ -226,9 +226,11 @@ def _stream_ptr(stream, device) -> int:
 
 
 def _check_frame(rgb, depth, H, W):
-    if rgb.shape[-3:] != (H, W, 3) or rgb.element_size() != 1:
+    # (a shape may be a list; the conversion is for those alone)
+    s, d = rgb.shape[-3:], depth.shape[-2:]
+    if (s != (H, W, 3) and tuple(s) != (H, W, 3)) or rgb.element_size() != 1:
         raise ValueError(f"rgb must be uint8 [{H}, {W}, 3]")
-    if depth.shape[-2:] != (H, W) or depth.element_size() != 2:
+    if (d != (H, W) and tuple(d) != (H, W)) or depth.element_size() != 2:
         raise ValueError(f"depth must be a 16-bit [{H}, {W}] tensor")
 
 
