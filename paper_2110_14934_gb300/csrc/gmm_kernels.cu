@@ -11,6 +11,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "gmm_internal.h"
 
 using namespace gmmdev;
@@ -79,15 +81,15 @@ __global__ void __launch_bounds__(256, (TickBounds<M, PREC, kLoop>::kCtas))
 
 // Runs per CTA. Looping saves CTA turnover and hides the next run's state
 // behind the current one, but leaves fewer CTAs to even out the end of the
-// launch: it pays from about a dozen waves of a GB300's 152 SMs x 1024
+// launch: it pays from about a dozen waves of the SMs x 1024
 // threads on. Measured (us; 1, 2, 4 runs): FP32 1280x720 M = 3 options 26.3,
 // 27.9, 30.1; 1920x1080 M = 5 63.6, 62.7, 64.3; 2560x1440 M = 4 95.8, 92.2,
 // 93.2; 3840x2160 M = 5 238, 227, 227; FP16/BF16 1920x1080 M = 3 35.5, 33.7,
 // 33.8; 2560x1440 M = 4 66.7, 64.6, 63.7; 3840x2160 M = 3 133.8, 117.6, 115.7;
 // M = 5 (whose looping form has 32 warps per SM against 40) 1920x1080 43.2,
 // 44.4, 44.7; 3840x2160 162.8, 154.6, 150.7.
-template <int M, int PREC> int tick_runs(int64_t n_pad) {
-    const int64_t waves = n_pad / (152 * 1024);
+template <int M, int PREC> int tick_runs(int64_t n_pad, int sms) {
+    const int64_t waves = n_pad / (sms * (int64_t)1024);
     if (waves >= 32)
         return 4;
     return waves >= (PREC != kF32 && M == 5 ? 20 : 12) ? 2 : 1;
@@ -99,16 +101,18 @@ cudaError_t launch_tick_v(const CamView &cv, int threads, cudaStream_t s) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    const int runs = tick_runs<M, PREC>(cv.n_pad);
+    const int sms = gmmhost::num_sms();
+    const int runs = tick_runs<M, PREC>(cv.n_pad, sms);
     const int64_t px = (int64_t)threads * runs;
-    // Two waves of CTAs. An opening's few CTAs leave HBM idle, and so does the
+    // 2560 threads per SM: two waves of CTAs, two and a half of the forms that
+    // keep 32 warps resident. An opening's few CTAs leave HBM idle, and so does the
     // end of a tick: with an opening after each tick FP32 1021x767 M = 4 26.7 ->
     // 25.2 us, 1280x720 M = 3 options 26.0 -> 25.1, caller-owned FP16/BF16
     // 1280x720 M = 4 22.1 -> 21.3; ticks alone FP32 1920x1080 M = 5 62.6 ->
     // 62.0. The FP16/BF16 handles' kernel loses by it (1920x1080 M = 5 43.1 ->
     // 46.5 us: more spills, and the state it would move is a smaller part of
     // its time), and does without.
-    const int early = 152 * 2560 / threads;
+    const int early = sms * 2560 / threads;
     cfg.gridDim = dim3((unsigned)((cv.n_pad + px - 1) / px));
     cfg.blockDim = dim3((unsigned)threads);
     cfg.stream = s;
@@ -348,12 +352,19 @@ cudaError_t launch_confusion(const uint32_t *pred, const uint32_t *truth, int H,
     return cudaGetLastError();
 }
 
+// SMs of the current device (asked for once per device).
 int num_sms() {
+    static std::atomic<int> known[64];
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess)
         return 1;
+    std::atomic<int> *slot = dev >= 0 && dev < 64 ? &known[dev] : nullptr;
+    if (slot && (n = slot->load(std::memory_order_relaxed)) > 0)
+        return n;
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return 1;
+    if (slot)
+        slot->store(n, std::memory_order_relaxed);
     return n;
 }
 
