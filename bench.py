@@ -842,8 +842,7 @@ def run_pool(args, wl):
                     "d2h_bytes_per_step": e2e["d2h"], "launch": e2e["launch"],
                     "path": "pinned packed tick-sets -> device staging (copy stream) -> "
                             "gmm_pool_submit_many + gmm_pool_tick -> masks to pinned host "
-                            "(FP16/BF16 prefetch off; the launch shape tuned in "
-                            "this pipeline unless fixed)"},
+                            "(the launch shape tuned in this pipeline unless fixed)"},
             "e2e_zero_copy": {"value": e2e["zero_copy"], "unit": UNIT,
                               "h2d_bytes_per_step": e2e["h2d"], "d2h_bytes_per_step": e2e["d2h"],
                               "launch": e2e["launch_zero_copy"],
@@ -1007,9 +1006,7 @@ def run_pool_e2e(G, torch, pool, ids, cams, frames, dev, stream, steps, warmup, 
     tick is packed into one pinned buffer, uploaded with one copy into one of
     two device staging buffers on a copy stream (overlapping the previous
     tick's compute), the pool ticks from there, and the packed masks come back
-    with one copy on a third stream, with the pool's FP16/BF16 next-tile
-    prefetch turned off (the library documents that uploads beside each tick
-    slow down under it). Then the zero-copy form, prefetch on. retune: the
+    with one copy on a third stream. Then the zero-copy form. retune: the
     pool's online tuner runs again inside each of the two pipelines before
     its warm-up (a shape's tick period then includes what its kernel delays
     in the uploads beside it, or in its own reads over the host link)."""
@@ -1071,7 +1068,6 @@ def run_pool_e2e(G, torch, pool, ids, cams, frames, dev, stream, steps, warmup, 
             shape["tuning_ticks"] = n
         return n, shape
 
-    pool.set_prefetch(False)
     k0, shape = tune(tick)
     for k in range(warmup):
         tick(k0 + k)
@@ -1095,7 +1091,6 @@ def run_pool_e2e(G, torch, pool, ids, cams, frames, dev, stream, steps, warmup, 
                          [mb_h + r * mask_bytes + m for m in moff])
         pool.tick(stream)
 
-    pool.set_prefetch(True)
     z0, shape_zc = tune(tick_zc)
     for k in range(warmup):
         tick_zc(z0 + k)

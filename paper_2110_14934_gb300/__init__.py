@@ -440,8 +440,7 @@ class Pool:
         _check(load_library().gmm_pool_use_graph(self._p, int(bool(enable))))
 
     def set_prefetch(self, enable=True) -> None:
-        """FP16/BF16 L2 prefetch (on by default); turn it off when
-        frames are uploaded on a copy stream beside every tick."""
+        """FP16/BF16 L2 prefetch (on by default)."""
         _check(load_library().gmm_pool_set_prefetch(self._p, int(bool(enable))))
 
     def state_get(self, cam, plane, component=0) -> np.ndarray:

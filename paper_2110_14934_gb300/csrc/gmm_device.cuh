@@ -98,8 +98,8 @@ __device__ __forceinline__ float var_sample(const StreamPrm &p, float d2) {
     return (p.flags & kVarPerChannel) ? d2 / (float)D : d2;
 }
 
-// Everything one tick of one camera needs; passed by value to the
-// single-camera kernel, read from constant memory by the pooled kernel.
+// Everything one tick of one camera needs: a parameter of the single-camera
+// kernel, one of up to 128 in those of the pooled kernels.
 struct CamView {
     void *planes;          // n_tiles tiles of M*8 planes of kTile elements
     uint8_t *fusion;       // n_tiles*kTile List-1 bytes, indexed by padded pixel
@@ -264,36 +264,9 @@ __device__ __forceinline__ int background_test(const float (&w)[M], int rank, bo
     }
     return (!matched || before > T) ? 1 : 0;
 }
-// One tick of one mixture without the whole state in hand. A tick changes every weight, and of the means and variances only those of the
-// component that matched or was replaced, unless components change places.
-// So it needs every weight and variance (the ranking) and the best-ranked
-// component's mean, which the caller has loaded; the other means are loaded
-// only in lanes that do not match the best-ranked component or whose
-// components change places, and only what changed is stored: of 16 M values
-// moved per pixel, 6 M + 10 remain for a background pixel. (Per-lane
-// predicates: a warp moves the 32-byte sectors its lanes ask for. A lane that
-// stores a mean or a variance has loaded that element, so a partly stored
-// sector is one the L2 already holds.) Measured in FP32 against moving the
-// whole state (HBM-bound at 100% of the copy bandwidth): one 1920x1080
-// camera, M = 5, 101.1 -> 64.7 us per tick (DRAM reads 108 instead of 165
-// bytes per pixel); 64 pooled cameras 2299 -> 1371 us. In FP16/BF16: 54.7 ->
-// 45.7 us, with the caller's layout (whose weights share a group with means)
-// 1280x720, M = 4, with opening 25.5 -> 23.3 us.
-//
-// Io is where the state lives: load_means(m, i0) fills this lane's stored
-// means m[i0..]; put(r, mu, v) takes the new mean and variance at rank r
-// (r known at compile time, only for ranks that changed). w, v: the weights
-// (updated to the new ones, in rank order) and variances; mu: the best-ranked
-// component's mean.
-// Returns the stream's foreground bit. lanes: the set of lanes of the warp that
-// make this same call, computed by the caller before the code diverged. Where
-// every lane of the call matches its best-ranked component (the usual case
-// for background pixels) the update is specialised to that; it computes
-// exactly what the general one does. The ranking is one copy of code for both,
-// and means are read again where components change places: with a ranking
-// per path the pooled FP16/BF16 kernel, which holds a body per M, spent a
-// third of its time on instruction fetch (24 cameras of odd sizes: 495 us
-// against 404; FP32 1920x1080 63.5 against 64.7).
+
+// The matched component's new mean (in place) and variance (returned), from its
+// variance v and the squared distance d2 to the old mean.
 template <int D, bool kOptions>
 __device__ __forceinline__ float moved_component(float (&mu)[D], float v, const float (&x)[D],
                                                  const StreamPrm &p, float d2) {
@@ -310,6 +283,38 @@ __device__ __forceinline__ float moved_component(float (&mu)[D], float v, const 
     return fmaxf(p.v_min, fmaf(orho, v, rho * (kOptions ? var_sample<D>(p, d2n) : d2n)));
 }
 
+// One tick of one mixture without the whole state in hand. A tick changes
+// every weight, and of the means and variances only those of the component that
+// matched or was replaced, unless components change places. So it needs every weight and variance (the ranking) and the best-ranked
+// component's mean, which the caller has loaded; the other means are loaded
+// only in lanes that do not match the best-ranked component or whose
+// components change places, and only what changed is stored: of 16 M values
+// moved per pixel, 6 M + 10 remain for a background pixel. (Per-lane
+// predicates: a warp moves the 32-byte sectors its lanes ask for. A lane that
+// stores a mean or a variance has loaded that element, so a partly stored
+// sector is one the L2 already holds.) Measured in FP32 against moving the
+// whole state (HBM-bound at 100% of the copy bandwidth), with the steps that
+// followed: one 1920x1080 camera, M = 5, 101.1 -> 62.0 us per tick (DRAM reads
+// 110 instead of 165 bytes per pixel); 64 pooled cameras 2294 -> 1266 us. In
+// FP16/BF16: 54.7 -> 44.2 us, with the caller's layout (whose weights share a
+// group with means) 1280x720, M = 4, with opening 25.5 -> 21.4 us. Frames in
+// which every pixel misses cost a second trip: noise at 1920x1080, M = 5, FP32
+// 101.5 -> 81.7 us, FP16/BF16 55.9 -> 58.0.
+//
+// Io is where the state lives: load_means(m, i0) fills this lane's stored
+// means m[i0..]; put(r, mu, v) takes the new mean and variance at rank r
+// (r known at compile time, only for ranks that changed). w, v: the weights
+// (updated to the new ones, in rank order) and variances; mu: the best-ranked
+// component's mean.
+// Returns the stream's foreground bit. lanes: the set of lanes of the warp that
+// make this same call, computed by the caller before the code diverged. Where
+// every lane of the call matches its best-ranked component (the usual case
+// for background pixels) the update is specialised to that; it computes
+// exactly what the general one does. The ranking is one copy of code for both,
+// and means are read again where components change places: with a ranking
+// per path the pooled FP16/BF16 kernel, which holds a body per M, spent a
+// third of its time on instruction fetch (24 cameras of odd sizes: 495 us
+// against 404; FP32 1920x1080 63.5 against 64.7).
 template <int M, int D, bool kOptions, bool kNormalV, class Io>
 __device__ __forceinline__ int ranked_step(Io &io, float (&w)[M], float (&v)[M], float (&mu)[D],
                                            const float (&x)[D], const StreamPrm &p,

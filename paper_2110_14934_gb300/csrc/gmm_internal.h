@@ -13,8 +13,8 @@ namespace gmmhost {
 cudaError_t launch_tick(const gmmdev::CamView &cv, int threads, cudaStream_t s);
 
 // Block size of the direct tick kernel for gmm_set_kernel's variant: 0 the
-// measured best for the storage precision (FP32: 128; FP16/BF16: 64, 45.7 us
-// against 46.4 with 128 at 1920x1080, M = 5), 1..4: 256, 128, 64, 32.
+// measured best for the storage precision (FP32: 128; FP16/BF16: 64, 1.5% faster
+// than 128 at 1920x1080, M = 5), 1..4: 256, 128, 64, 32.
 inline int direct_threads(int variant, int prec) {
     switch (variant) {
     case 1: return 256;
@@ -55,8 +55,8 @@ cudaError_t launch_morph_open3(const uint32_t *in, uint32_t *out, int H, int W,
 // [tile_begin[j], tile_begin[j+1]) of camera views[j], tile_pixels pixels
 // each (the last one of a camera ragged). A launch handles up to kPoolViews
 // cameras (a tick with more is split into several launches); its PoolArgs
-// are the kernel's parameters. *counter must be zero at launch; the launch zeroes the n_reset
-// counters at reset (the next tick's).
+// are the kernel's parameters. *counter must be zero at launch; the launch
+// zeroes the n_reset counters at reset (the next tick's).
 constexpr int kPoolViews = 128;
 struct PoolArgs {
     gmmdev::CamView views[kPoolViews];
@@ -70,12 +70,11 @@ struct PoolArgs {
 };
 static_assert(sizeof(PoolArgs) <= 32764, "one launch's arguments fit the kernel parameters");
 
-// Launch the pool kernel; all_variants: the instance
-// that also handles the options and the augmentation alternative; flat: the
-// non-persistent form (tile_begin and n_tiles count one chunk per warp:
-// 32 pixels in FP32, 64 in FP16/BF16; blocks covers every chunk); m: the M
-// every camera of the launch has (a kernel specialised to it), or 0;
-// prefetch: the FP16/BF16 persistent instance that prefetches each warp's next
+// Launch the pool kernel; all_variants: the instance that also handles the
+// options and the augmentation alternative; flat: the non-persistent form
+// (tile_begin and n_tiles count one chunk per warp: 32 pixels in FP32, 64 in
+// FP16/BF16; blocks covers every chunk); m: the M every camera of the launch
+// has (a kernel specialised to it), or 0; prefetch: the FP16/BF16 persistent instance that prefetches each warp's next
 // pixels into L2 (else the one that does not).
 cudaError_t launch_pool_tick_impl(const PoolArgs &args, int threads, int blocks, int prec,
                                   bool all_variants, bool flat, int m, bool prefetch,

@@ -81,8 +81,7 @@ __global__ void __launch_bounds__(256, (TickBounds<M, PREC, kLoop>::kCtas))
 
 // Runs per CTA. Looping saves CTA turnover and hides the next run's state
 // behind the current one, but leaves fewer CTAs to even out the end of the
-// launch: it pays from about a dozen waves of the SMs x 1024
-// threads on. Measured (us; 1, 2, 4 runs): FP32 1280x720 M = 3 options 26.3,
+// launch: it pays from about a dozen waves of the SMs x 1024 threads on. Measured (us; 1, 2, 4 runs): FP32 1280x720 M = 3 options 26.3,
 // 27.9, 30.1; 1920x1080 M = 5 63.6, 62.7, 64.3; 2560x1440 M = 4 95.8, 92.2,
 // 93.2; 3840x2160 M = 5 238, 227, 227; FP16/BF16 1920x1080 M = 3 35.5, 33.7,
 // 33.8; 2560x1440 M = 4 66.7, 64.6, 63.7; 3840x2160 M = 3 133.8, 117.6, 115.7;
@@ -105,8 +104,8 @@ cudaError_t launch_tick_v(const CamView &cv, int threads, cudaStream_t s) {
     const int runs = tick_runs<M, PREC>(cv.n_pad, sms);
     const int64_t px = (int64_t)threads * runs;
     // 2560 threads per SM: two waves of CTAs, two and a half of the forms that
-    // keep 32 warps resident. An opening's few CTAs leave HBM idle, and so does the
-    // end of a tick: with an opening after each tick FP32 1021x767 M = 4 26.7 ->
+    // keep 32 warps resident. An opening's few CTAs leave HBM idle, and so does
+    // the end of a tick: with an opening after each tick FP32 1021x767 M = 4 26.7 ->
     // 25.2 us, 1280x720 M = 3 options 26.0 -> 25.1, caller-owned FP16/BF16
     // 1280x720 M = 4 22.1 -> 21.3; ticks alone FP32 1920x1080 M = 5 62.6 ->
     // 62.0. The FP16/BF16 handles' kernel loses by it (1920x1080 M = 5 43.1 ->

@@ -81,7 +81,7 @@ __device__ __forceinline__ int tile_job(const PoolArgs &a, int64_t t) {
 // 842 on 64 FP16/BF16 cameras, each at its best launch shape, now that a tile
 // prefetches within itself.)
 template <int PREC, bool kAll, bool kPF>
-__global__ void __launch_bounds__(256, PREC == 0 && kAll ? 3 : 4) 
+__global__ void __launch_bounds__(256, PREC == 0 && kAll ? 3 : 4)
     k_pool_tick(const __grid_constant__ PoolArgs a) {
     dependent_launch_prologue();
     __shared__ int64_t s_tile;
@@ -114,8 +114,7 @@ __global__ void __launch_bounds__(256, PREC == 0 && kAll ? 3 : 4)
 // Non-persistent form: every warp takes one chunk of the launch's implicit
 // chunk list (tile_begin counts chunks here: 32 pixels in FP32, one per lane;
 // 64 in FP16/BF16, two per lane with the second pixel's loads overlapping
-// the first one's arithmetic, as in the single-camera kernels) and finds its
-// camera by binary search. No counter and no loop: a CTA's slot frees as soon
+// the first one's arithmetic) and finds its camera by binary search. No counter and no loop: a CTA's slot frees as soon
 // as its own warps finish, and no registers carry a loop across pixels.
 template <int M, int PREC, int V>
 __device__ __forceinline__ void flat_chunk(const CamView &cv, int64_t base) {
@@ -155,7 +154,7 @@ __device__ __forceinline__ void flat_chunk_v(const CamView &cv, int64_t base) {
 // (any M, switched per warp). FP32: no residency hint; FP16/BF16: 64
 // registers, as in the other kernels.
 template <int PREC, bool kAll, int MM>
-__global__ void __launch_bounds__(256, PREC == 0 ? 1 : 4) 
+__global__ void __launch_bounds__(256, PREC == 0 ? 1 : 4)
     k_pool_flat(const __grid_constant__ PoolArgs a) {
     dependent_launch_prologue();
     if (blockIdx.x == 0) // the next tick's counters, as the persistent form does

@@ -219,7 +219,7 @@ static cudaError_t enqueue_tick(gmm_server *s, TickRec &t) {
 // the cap 0.42 and 1.6). In the copy mode a tick's uploads, kernel and downloads
 // run on three streams and the next tick's uploads start as soon as the last
 // one's are done, so nothing is held back there (the same cameras: p50 0.46-0.50
-// ms, p99 4.0-4.6; with two ticks 1.9 and 9.9-11.1, with three 1.4 and 9.7-9.9).
+// ms, p99 4.0-6.9; with two ticks 1.9 and 9.9-11.1, with three 1.4 and 9.7-9.9).
 constexpr size_t kTicksInFlight = 2;
 
 static void engine_main(gmm_server *s) {
