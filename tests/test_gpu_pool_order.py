@@ -5,6 +5,7 @@ camera's admission and release, state reads, the host's wait. The stream of the
 earlier work is held back by other work, so that later work that did not wait
 would overtake it; the results equal a pool that keeps to one stream."""
 import ctypes
+import itertools
 import queue
 import threading
 
@@ -29,26 +30,31 @@ class Handle:
 
 @pytest.fixture(scope="module")
 def setup():
-    """Frames, and what holds a stream back: some 4 ms of full-HD ticks."""
+    """Frames, and what holds a stream back: some 4 ms of full-HD ticks, on a
+    model of their own at each call (four in turn; a test waits for the GPU
+    before it makes a fifth)."""
     import torch
     rgb, depth, _ = scene_frames(81, H, W, 1, 44, N)
     frames = [to_dev(r, d) for r, d in zip(rgb, depth)]
-    big = G.GMM(1080, 1920, 5)
+    models = [G.GMM(1080, 1920, 3) for _ in range(4)]
+    masks = [g.new_mask() for g in models]
+    turn = itertools.cycle(zip(models, masks))
     br, bd = (torch.zeros(s, dtype=t, device="cuda") for s, t in (((1080, 1920, 3), torch.uint8), ((1080, 1920), torch.int16)))
-    bm = big.new_mask()
 
     def hold(stream):
-        for _ in range(60):
-            big.apply(br, bd, bm, stream=stream)
+        g, m = next(turn)
+        for _ in range(100):
+            g.apply(br, bd, m, stream=stream)
 
     torch.cuda.synchronize()
     yield frames, hold
     torch.cuda.synchronize()
-    big.set_stream(torch.cuda.default_stream())
-    big.close()
+    for g in models:
+        g.set_stream(torch.cuda.default_stream())
+        g.close()
 
 
-def _run(frames, tick, before_close=None):
+def _run(frames, tick):
     """Masks of every tick and the final state of a pool of one camera."""
     import torch
     p = G.Pool()
